@@ -206,6 +206,10 @@ struct pmc_chains_s {
   double* d_z2 = nullptr;
   std::vector<double> h_z2;        // host copy of d_z2 (filled at the first estimate)
   double* d_est = nullptr;         // per-pair moments [n_pairs][PMC_MOMENT_WORDS]
+  int n_mom_chunks = 0, n_mom_pairs = 0;  // chunks of the moment reduction, pairs of several chunks
+  MomChunk* d_mom_chunks = nullptr;
+  MomPair* d_mom_pairs = nullptr;
+  double* d_mom_part = nullptr;    // partial sums per chunk
   long long chain_lo = 0;          // this set holds the geometry's chains [chain_lo, chain_lo + total)
   int* h_abort = nullptr;
   int* d_abort = nullptr;
@@ -590,6 +594,9 @@ int pmc_destroy_chains(pmc_chains_t ch) {
   cudaFree(ch->d_queue);
   cudaFree(ch->d_z2);
   cudaFree(ch->d_est);
+  cudaFree(ch->d_mom_chunks);
+  cudaFree(ch->d_mom_pairs);
+  cudaFree(ch->d_mom_part);
   cudaFree(ch->d_stage);
   cudaFree(ch->d_stage_n);
   cudaFree(ch->d_qp);
@@ -1032,6 +1039,20 @@ int pmc_init_chains(pmc_ctx_t ctx, pmc_medium_t med, pmc_geom_t geom, const pmc_
   CK(dalloc(&ch->d_queue, ch->classes.size()));
   CK(dalloc(&ch->d_z2, ch->n_pairs));
   CK(dalloc(&ch->d_est, static_cast<size_t>(ch->n_pairs) * PMC_MOMENT_WORDS));
+  std::vector<MomChunk> mom_chunks;
+  std::vector<MomPair> mom_pairs;
+  for (int p = 0; p < ch->n_pairs; ++p) {
+    const DPair& d = ch->h_pairs[p];
+    const int n_chunks = std::max(1, (d.n_chains + kMomChunk - 1) / kMomChunk);
+    if (n_chunks > 1) mom_pairs.push_back({p, static_cast<int>(mom_chunks.size()), n_chunks});
+    for (int k = 0; k < n_chunks; ++k)
+      mom_chunks.push_back({p, d.chain0 + k * kMomChunk, std::min(kMomChunk, d.n_chains - k * kMomChunk), n_chunks == 1});
+  }
+  ch->n_mom_chunks = static_cast<int>(mom_chunks.size());
+  ch->n_mom_pairs = static_cast<int>(mom_pairs.size());
+  CK(dalloc(&ch->d_mom_chunks, mom_chunks.size()));
+  CK(dalloc(&ch->d_mom_pairs, mom_pairs.size()));
+  CK(dalloc(&ch->d_mom_part, mom_pairs.empty() ? 1 : mom_chunks.size() * MOM_USED));
   if (ch->lam_on) {
     const int K = R.n_spec;
     std::vector<float> spec(2 * static_cast<size_t>(K));
@@ -1055,6 +1076,8 @@ int pmc_init_chains(pmc_ctx_t ctx, pmc_medium_t med, pmc_geom_t geom, const pmc_
   CK(cudaMemcpyAsync(ch->d_chain_pair, ch->h_pair_of.data(), sizeof(int) * T, cudaMemcpyHostToDevice, s));
   CK(cudaMemcpyAsync(ch->d_chain_base, ch->h_base.data(), sizeof(long long) * T, cudaMemcpyHostToDevice, s));
   CK(cudaMemcpyAsync(ch->d_order, order.data(), sizeof(int) * T, cudaMemcpyHostToDevice, s));
+  CK(cudaMemcpyAsync(ch->d_mom_chunks, mom_chunks.data(), sizeof(MomChunk) * mom_chunks.size(), cudaMemcpyHostToDevice, s));
+  CK(cudaMemcpyAsync(ch->d_mom_pairs, mom_pairs.data(), sizeof(MomPair) * mom_pairs.size(), cudaMemcpyHostToDevice, s));
   CK(cudaMemsetAsync(ch->d_status, 0, sizeof(int) * T, s));
   CK(cudaMemsetAsync(ch->d_any, 0, sizeof(int), s));
   CK(cudaMemsetAsync(ch->d_xyz, 0, sizeof(float) * ch->xyz_floats, s));
@@ -1253,7 +1276,8 @@ static int read_moments(pmc_chains_t ch, std::vector<double>& h, cudaStream_t s)
     ch->h_z2.resize(ch->n_pairs);
     CK(cudaMemcpyAsync(ch->h_z2.data(), ch->d_z2, sizeof(double) * ch->n_pairs, cudaMemcpyDeviceToHost, s));
   }
-  CK(launch_moments(ch->d_acc, ch->d_pairs, ch->n_pairs, moments_ls(ch), moments_la(ch), ch->d_est, s));
+  CK(launch_moments(ch->d_acc, ch->d_mom_chunks, ch->n_mom_chunks, ch->d_mom_pairs, ch->n_mom_pairs, moments_ls(ch),
+                    moments_la(ch), ch->d_mom_part, ch->d_est, s));
   h.resize(static_cast<size_t>(ch->n_pairs) * PMC_MOMENT_WORDS);
   CK(cudaMemcpyAsync(h.data(), ch->d_est, h.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
   return check_status(ch, s);

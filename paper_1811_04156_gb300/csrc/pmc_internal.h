@@ -177,10 +177,21 @@ __host__ __device__ inline void add_chain_moments(const double* acc, double ls, 
   }
 }
 
-// Per-pair moments of the chains' accumulators (one block per pair, FP64):
-// out[n_pairs][PMC_MOMENT_WORDS].
-cudaError_t launch_moments(const double* acc, const DPair* pairs, int n_pairs, double ls, double la, double* out,
-                           cudaStream_t s);
+// Per-pair moments of the chains' accumulators (FP64): out[n_pairs][PMC_MOMENT_WORDS].
+// The chains are split into chunks of at most kMomChunk chains of one pair
+// (every pair has at least one, an empty one if a chain window leaves it no
+// chains); pairs of several chunks are listed in `pairs` and go through the
+// partial sums part[n_chunks][MOM_USED].
+constexpr int kMomChunk = 128;
+struct MomChunk {
+  int pair, first, n;           // chains [first, first + n) of pair `pair`
+  int last;                     // 1: the pair's only chunk
+};
+struct MomPair {
+  int pair, first, n;           // chunks [first, first + n) of pair `pair`
+};
+cudaError_t launch_moments(const double* acc, const MomChunk* chunks, int n_chunks, const MomPair* pairs, int n_pairs,
+                           double ls, double la, double* part, double* out, cudaStream_t s);
 // Estimate of one pair from its moments (host; pmc_estimate_from_moments).
 void estimate_of_moments(const double* mom, double z2, pmc_estimate* out, double* grad, double* grad_se);
 

@@ -199,22 +199,82 @@ __global__ void __launch_bounds__(256) z2_kernel(const DMedium M, const DPair* _
   if (threadIdx.x == 0) out[blockIdx.x] = vv[0];
 }
 
-// Per-pair moments of the chain accumulators (one block per pair): sums
-// over the pair's chains, each chain's terms from add_chain_moments.
-__global__ void __launch_bounds__(256) moments_kernel(const double* __restrict__ acc, const DPair* __restrict__ pairs,
-                                                      double ls, double la, double* __restrict__ out) {
-  __shared__ double sh[8 * MOM_USED];
-  const DPair S = pairs[blockIdx.x];
+// Sum over the warp's lanes of each of `K` values (K a power of two, at most
+// 32) by recursive halving: at every step a lane hands half of its values to
+// its partner and adds the partner's copy of the other half, so that K values
+// cost K - 1 + log2(32 / K) additions per lane instead of the 5 K of a
+// butterfly.  Afterwards v[0] of a lane is the warp's total of the value whose
+// index is the lane's top log2(K) bits.
+template <int K>
+__device__ __forceinline__ void warp_scatter_sum(double* v, int lane) {
+  int o = 16;
+#pragma unroll
+  for (int m = K; m > 1; m >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int k = 0; k < m / 2; ++k) {
+      const double give = up ? v[k] : v[k + m / 2];
+      const double keep = up ? v[k + m / 2] : v[k];
+      v[k] = keep + __shfl_xor_sync(kFull, give, o);
+    }
+  }
+  for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(kFull, v[0], o);
+}
+
+// Per-pair moments of the chain accumulators, first pass: one block per chunk
+// of at most kMomChunk chains of one pair, one chain per thread, each chain's
+// terms from add_chain_moments.  A pair of one chunk is finished here, the
+// partial sums of the others go to part[chunk][MOM_USED].
+//
+// Bound by the FP64 pipe (about 80 FP64 operations per chain): with one block
+// per pair a single pair of 65,536 chains kept one SM busy for 1,359 us; in
+// chunks of 128 chains over all SMs (and 51 additions per lane for the
+// block's sums instead of 180) both passes take 27 us.
+__global__ void __launch_bounds__(kMomChunk) moments_kernel(const double* __restrict__ acc,
+                                                            const MomChunk* __restrict__ chunks, double ls, double la,
+                                                            double* __restrict__ part, double* __restrict__ out) {
+  constexpr int kWarps = kMomChunk / 32;
+  __shared__ double sh[kWarps][MOM_USED];
+  const MomChunk C = chunks[blockIdx.x];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   double v[MOM_USED];
 #pragma unroll
   for (int k = 0; k < MOM_USED; ++k) v[k] = 0.0;
-  for (int c = S.chain0 + threadIdx.x; c < S.chain0 + S.n_chains; c += blockDim.x)
-    add_chain_moments(acc + static_cast<size_t>(c) * ACC_WORDS, ls, la, v);
-  block_sum<MOM_USED>(v, sh);
-  if (threadIdx.x != 0) return;
-  double* o = out + static_cast<size_t>(blockIdx.x) * PMC_MOMENT_WORDS;
-#pragma unroll
-  for (int k = 0; k < PMC_MOMENT_WORDS; ++k) o[k] = k < MOM_USED ? v[k] : 0.0;
+  if (static_cast<int>(threadIdx.x) < C.n)
+    add_chain_moments(acc + static_cast<size_t>(C.first + threadIdx.x) * ACC_WORDS, ls, la, v);
+  static_assert(MOM_USED == 36, "32 + 4 values");
+  warp_scatter_sum<32>(v, lane);
+  sh[w][lane] = v[0];
+  warp_scatter_sum<4>(v + 32, lane);
+  if ((lane & 7) == 0) sh[w][32 + (lane >> 3)] = v[32];
+  __syncthreads();
+  const int k = threadIdx.x;
+  if (k >= PMC_MOMENT_WORDS) return;
+  double x = 0.0;
+  if (k < MOM_USED)
+    for (int i = 0; i < kWarps; ++i) x += sh[i][k];
+  if (C.last) out[static_cast<size_t>(C.pair) * PMC_MOMENT_WORDS + k] = x;
+  else if (k < MOM_USED) part[static_cast<size_t>(blockIdx.x) * MOM_USED + k] = x;
+}
+
+// Second pass: one block per pair of several chunks, kMomGroups groups of
+// threads over the pair's partial sums.
+constexpr int kMomGroups = 8;
+__global__ void __launch_bounds__(kMomGroups * MOM_USED) moments_total_kernel(const double* __restrict__ part,
+                                                                              const MomPair* __restrict__ pairs,
+                                                                              double* __restrict__ out) {
+  __shared__ double sh[kMomGroups][MOM_USED];
+  const MomPair C = pairs[blockIdx.x];
+  const int g = threadIdx.x / MOM_USED, k = threadIdx.x % MOM_USED;
+  double x = 0.0;
+  for (int i = g; i < C.n; i += kMomGroups) x += part[static_cast<size_t>(C.first + i) * MOM_USED + k];
+  sh[g][k] = x;
+  __syncthreads();
+  if (threadIdx.x >= PMC_MOMENT_WORDS) return;
+  x = 0.0;
+  if (threadIdx.x < MOM_USED)
+    for (int i = 0; i < kMomGroups; ++i) x += sh[i][threadIdx.x];
+  out[static_cast<size_t>(C.pair) * PMC_MOMENT_WORDS + threadIdx.x] = x;
 }
 
 // ---------------------------------------------------------------------------
@@ -373,10 +433,11 @@ cudaError_t launch_z2(const DMedium& M, const DPair* pairs, int n_pairs, int n_v
   return cudaGetLastError();
 }
 
-cudaError_t launch_moments(const double* acc, const DPair* pairs, int n_pairs, double ls, double la, double* out,
-                           cudaStream_t s) {
-  if (n_pairs <= 0) return cudaSuccess;
-  moments_kernel<<<n_pairs, 256, 0, s>>>(acc, pairs, ls, la, out);
+cudaError_t launch_moments(const double* acc, const MomChunk* chunks, int n_chunks, const MomPair* pairs, int n_pairs,
+                           double ls, double la, double* part, double* out, cudaStream_t s) {
+  if (n_chunks <= 0) return cudaSuccess;
+  moments_kernel<<<n_chunks, kMomChunk, 0, s>>>(acc, chunks, ls, la, part, out);
+  if (n_pairs > 0) moments_total_kernel<<<n_pairs, kMomGroups * MOM_USED, 0, s>>>(part, pairs, out);
   return cudaGetLastError();
 }
 
