@@ -132,9 +132,12 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1
   return c;
 }
 
-// ((x >> 9) + 1/2) * 2^-23: exact in FP32, in (0, 1).
+// ((x >> 9) + 1/2) * 2^-23: exact in FP32, in (0, 1).  The 23 bits become the
+// mantissa of a float in [1, 2), from which 1 - 2^-24 is subtracted (exact:
+// the difference is an odd multiple of 2^-24 below 1), so no integer-to-float
+// conversion runs on the quarter-rate unit.
 __device__ __forceinline__ float u01(uint32_t x) {
-  return __fmaf_rn(static_cast<float>(x >> 9), 1.1920928955078125e-7f, 5.9604644775390625e-8f);
+  return __fadd_rn(__uint_as_float((x >> 9) + 0x3f800000u), -0.999999940395355224609375f);
 }
 // floor(23-bit fraction * m), in integers.
 __device__ __forceinline__ uint32_t index_draw(uint32_t x, uint32_t m) {

@@ -1,5 +1,7 @@
 // Density, adjoint, score, normalisation, estimator and forward-tracer kernels
 // (Collin, arXiv:1811.04156).
+#include <algorithm>
+
 #include "pmc_internal.h"
 #include "pmc_tracer.cuh"
 
@@ -278,34 +280,40 @@ __global__ void __launch_bounds__(kMomGroups * MOM_USED) moments_total_kernel(co
 }
 
 // ---------------------------------------------------------------------------
-// Forward tracer (appendix, "Ray tracer"; the photon itself in pmc_tracer.cuh):
+// Forward tracer (appendix, "Ray tracer"; the photons in pmc_tracer.cuh):
 // one thread per photon.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) trace_kernel(const DMedium M, const DPair S, unsigned long long seed,
-                                                    unsigned long long photon0, unsigned long long n_photons,
-                                                    float r_reject, int max_scatter, double* __restrict__ out5,
-                                                    double* __restrict__ hist, double l_lo, double bins_per_m,
-                                                    int n_bins) {
+// Grid of the tracer kernels: 16 blocks per SM (3 or 4 are resident), so that
+// several waves even out the ends of the blocks: 8e6 lean photons took 16.5 ms
+// with 4 per SM, 15.7 with 8, 15.4 with 16; two-sensor photons 34.6, 30.8, 30.1.
+static unsigned trace_grid(unsigned long long n_photons, int n_sm) {
+  return static_cast<unsigned>(std::min((n_photons + 255) / 256, static_cast<unsigned long long>(n_sm) * 16ull));
+}
+
+template <bool kLean>
+__global__ void __launch_bounds__(256)
+    trace_kernel(const DMedium M, const DPair S, unsigned long long seed, unsigned long long photon0,
+                 unsigned long long n_photons, float r_reject, int max_scatter, double* __restrict__ out5,
+                 double* __restrict__ hist, double l_lo, double bins_per_m, int n_bins) {
   __shared__ double sh[8 * 5];
   const uint32_t k0 = static_cast<uint32_t>(seed), k1 = static_cast<uint32_t>(seed >> 32);
   double v[5] = {0, 0, 0, 0, 0};
-  const unsigned long long stride = static_cast<unsigned long long>(gridDim.x) * blockDim.x;
-  for (unsigned long long q = blockIdx.x * blockDim.x + threadIdx.x; q < n_photons; q += stride) {
-    const PhotonResult pr = trace_photon<false>(M, S, k0, k1, photon0 + q, r_reject, max_scatter, nullptr, nullptr,
-                                                nullptr);
-    v[3] += 1.0;
-    if (pr.hit) {
-      const double W = static_cast<double>(expf(pr.lw));
-      v[0] += W;
-      v[1] += W * W;
-      v[2] += 1.0;
-      v[4] += W * static_cast<double>(pr.L);
-      if (hist != nullptr) {
-        const double fb = (static_cast<double>(pr.L) - l_lo) * bins_per_m;
-        if (fb >= 0.0 && fb < static_cast<double>(n_bins)) atomicAdd(hist + static_cast<int>(fb), W);
-      }
-    }
-  }
+  unsigned int emitted = 0;
+  trace_photons<kLean>(M, S, k0, k1, photon0, n_photons, r_reject, max_scatter,
+                [&](unsigned long long, const PhotonResult& pr) {
+                  if (++emitted == 0u) v[3] += 4294967296.0;
+                  if (!pr.hit) return;
+                  const double W = static_cast<double>(expf(pr.lw));
+                  v[0] += W;
+                  v[1] += W * W;
+                  v[2] += 1.0;
+                  v[4] += W * static_cast<double>(pr.L);
+                  if (hist != nullptr) {
+                    const double fb = (static_cast<double>(pr.L) - l_lo) * bins_per_m;
+                    if (fb >= 0.0 && fb < static_cast<double>(n_bins)) atomicAdd(hist + static_cast<int>(fb), W);
+                  }
+                });
+  v[3] += static_cast<double>(emitted);
   block_sum<5>(v, sh);
   if (threadIdx.x == 0) {
 #pragma unroll
@@ -317,24 +325,21 @@ __global__ void __launch_bounds__(256) trace_kernel(const DMedium M, const DPair
 // exact draw from the normalised path density (cap-truncated by max_scatter).
 // Accepted paths are written to out_xyz [3][max_paths][stride] (absolute) and
 // out_n; *count counts every accepted path (also those beyond max_paths).
-__global__ void __launch_bounds__(256) trace_paths_kernel(const DMedium M, const DPair S, unsigned long long seed,
-                                                          unsigned long long photon0, unsigned long long n_photons,
-                                                          float r_reject, int max_scatter, int max_paths, int stride,
-                                                          float* __restrict__ out_xyz, int* __restrict__ out_n,
-                                                          unsigned int* __restrict__ count) {
+__global__ void __launch_bounds__(256)
+    trace_paths_kernel(const DMedium M, const DPair S, unsigned long long seed, unsigned long long photon0,
+                       unsigned long long n_photons, float r_reject, int max_scatter, int max_paths, int stride,
+                       float* __restrict__ out_xyz, int* __restrict__ out_n, unsigned int* __restrict__ count) {
   const uint32_t k0 = static_cast<uint32_t>(seed), k1 = static_cast<uint32_t>(seed >> 32);
-  const unsigned long long gstride = static_cast<unsigned long long>(gridDim.x) * blockDim.x;
   const size_t plane = static_cast<size_t>(max_paths) * stride;
-  for (unsigned long long q = blockIdx.x * blockDim.x + threadIdx.x; q < n_photons; q += gstride) {
-    const PhotonResult pr = trace_photon<false>(M, S, k0, k1, photon0 + q, r_reject, max_scatter, nullptr, nullptr,
-                                                nullptr);
-    if (!pr.hit || !(pr.u_acc < expf(pr.lw))) continue;
-    const unsigned int slot = atomicAdd(count, 1u);
-    if (slot >= static_cast<unsigned int>(max_paths)) continue;
-    float* ox = out_xyz + static_cast<size_t>(slot) * stride;
-    trace_photon<true>(M, S, k0, k1, photon0 + q, r_reject, max_scatter, ox, ox + plane, ox + 2 * plane);
-    out_n[slot] = pr.nsc + 2;
-  }
+  trace_photons<false>(M, S, k0, k1, photon0, n_photons, r_reject, max_scatter,
+                [&](unsigned long long ph, const PhotonResult& pr) {
+                  if (!pr.hit || !(pr.u_acc < expf(pr.lw))) return;
+                  const unsigned int slot = atomicAdd(count, 1u);
+                  if (slot >= static_cast<unsigned int>(max_paths)) return;
+                  float* ox = out_xyz + static_cast<size_t>(slot) * stride;
+                  record_photon<false>(M, S, k0, k1, ph, r_reject, max_scatter, ox, ox + plane, ox + 2 * plane);
+                  out_n[slot] = pr.nsc + 2;
+                });
 }
 
 // Per-layer scores of every chain's current path, summed per pair (layered
@@ -447,10 +452,8 @@ cudaError_t launch_trace(const DMedium& M, const DPair& S, unsigned long long se
   cudaError_t e = cudaMemsetAsync(out5, 0, 5 * sizeof(double), s);
   if (e != cudaSuccess) return e;
   if (n_photons == 0) return cudaSuccess;
-  unsigned long long blocks = (n_photons + 255) / 256;
-  const unsigned long long maxb = static_cast<unsigned long long>(n_sm) * 8ull;
-  if (blocks > maxb) blocks = maxb;
-  trace_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(M, S, seed, photon0, n_photons, r_reject,
+  const auto kernel = trace_lean(M, S) ? trace_kernel<true> : trace_kernel<false>;
+  kernel<<<trace_grid(n_photons, n_sm), 256, 0, s>>>(M, S, seed, photon0, n_photons, r_reject,
                                                              max_scatter, out5, nullptr, 0.0, 0.0, 0);
   return cudaGetLastError();
 }
@@ -463,10 +466,8 @@ cudaError_t launch_trace_lengths(const DMedium& M, const DPair& S, unsigned long
   if (e == cudaSuccess) e = cudaMemsetAsync(hist, 0, static_cast<size_t>(n_bins) * sizeof(double), s);
   if (e != cudaSuccess) return e;
   if (n_photons == 0) return cudaSuccess;
-  unsigned long long blocks = (n_photons + 255) / 256;
-  const unsigned long long maxb = static_cast<unsigned long long>(n_sm) * 8ull;
-  if (blocks > maxb) blocks = maxb;
-  trace_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(M, S, seed, photon0, n_photons, r_reject,
+  const auto kernel = trace_lean(M, S) ? trace_kernel<true> : trace_kernel<false>;
+  kernel<<<trace_grid(n_photons, n_sm), 256, 0, s>>>(M, S, seed, photon0, n_photons, r_reject,
                                                              max_scatter, out5, hist, l_lo,
                                                              static_cast<double>(n_bins) / (l_hi - l_lo), n_bins);
   return cudaGetLastError();
@@ -487,20 +488,18 @@ cudaError_t launch_layer_scores(const DMedium& M, const DPair* pairs, const int*
 // photon0 + n_photons) whose detection survives the thinning by w rho (the
 // same test as trace_paths_kernel), in any order, into idx[0 .. cap_idx);
 // *count receives how many there were (also beyond cap_idx).
-__global__ void __launch_bounds__(256) seed_count_kernel(const DMedium M, const DPair S, unsigned long long seed,
-                                                         unsigned long long photon0, unsigned long long n_photons,
-                                                         float r_reject, int max_scatter,
-                                                         unsigned long long* __restrict__ idx, unsigned int cap_idx,
-                                                         unsigned int* __restrict__ count) {
+template <bool kLean>
+__global__ void __launch_bounds__(256)
+    seed_count_kernel(const DMedium M, const DPair S, unsigned long long seed, unsigned long long photon0,
+                      unsigned long long n_photons, float r_reject, int max_scatter,
+                      unsigned long long* __restrict__ idx, unsigned int cap_idx, unsigned int* __restrict__ count) {
   const uint32_t k0 = static_cast<uint32_t>(seed), k1 = static_cast<uint32_t>(seed >> 32);
-  const unsigned long long gstride = static_cast<unsigned long long>(gridDim.x) * blockDim.x;
-  for (unsigned long long q = blockIdx.x * blockDim.x + threadIdx.x; q < n_photons; q += gstride) {
-    const PhotonResult pr = trace_photon<false>(M, S, k0, k1, photon0 + q, r_reject, max_scatter, nullptr, nullptr,
-                                                nullptr);
-    if (!pr.hit || !(pr.u_acc < expf(pr.lw))) continue;
-    const unsigned int slot = atomicAdd(count, 1u);
-    if (slot < cap_idx) idx[slot] = photon0 + q;
-  }
+  trace_photons<kLean>(M, S, k0, k1, photon0, n_photons, r_reject, max_scatter,
+                [&](unsigned long long ph, const PhotonResult& pr) {
+                  if (!pr.hit || !(pr.u_acc < expf(pr.lw))) return;
+                  const unsigned int slot = atomicAdd(count, 1u);
+                  if (slot < cap_idx) idx[slot] = ph;
+                });
 }
 
 // Chain seeding, second pass: chain chain0 + i of pair S (i < n) takes the
@@ -517,8 +516,7 @@ __global__ void __launch_bounds__(128) seed_record_kernel(const DMedium M, DPair
   S.org[0] = S.org[1] = S.org[2] = 0.f;  // record frame coordinates
   const uint32_t k0 = static_cast<uint32_t>(seed), k1 = static_cast<uint32_t>(seed >> 32);
   float* gx = xyz + chain_base[c];
-  const PhotonResult pr = trace_photon<true>(M, S, k0, k1, sel[i], r_reject, S.cap - 2, gx, gx + S.cap,
-                                             gx + 2 * S.cap);
+  const PhotonResult pr = record_photon<false>(M, S, k0, k1, sel[i], r_reject, S.cap - 2, gx, gx + S.cap, gx + 2 * S.cap);
   nv[c] = pr.hit ? pr.nsc + 2 : 2;
   status[c] = pr.hit ? 0 : ST_BAD_N;
 }
@@ -527,10 +525,8 @@ cudaError_t launch_seed_count(const DMedium& M, const DPair& S, unsigned long lo
                               unsigned long long n_photons, float r_reject, int max_scatter, unsigned long long* idx,
                               unsigned int cap_idx, unsigned int* count, int n_sm, cudaStream_t s) {
   if (n_photons == 0) return cudaSuccess;
-  unsigned long long blocks = (n_photons + 255) / 256;
-  const unsigned long long maxb = static_cast<unsigned long long>(n_sm) * 8ull;
-  if (blocks > maxb) blocks = maxb;
-  seed_count_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(M, S, seed, photon0, n_photons, r_reject,
+  const auto kernel = trace_lean(M, S) ? seed_count_kernel<true> : seed_count_kernel<false>;
+  kernel<<<trace_grid(n_photons, n_sm), 256, 0, s>>>(M, S, seed, photon0, n_photons, r_reject,
                                                                   max_scatter, idx, cap_idx, count);
   return cudaGetLastError();
 }
@@ -548,10 +544,7 @@ cudaError_t launch_trace_paths(const DMedium& M, const DPair& S, unsigned long l
                                unsigned long long n_photons, float r_reject, int max_scatter, int max_paths, int stride,
                                float* out_xyz, int* out_n, unsigned int* count, int n_sm, cudaStream_t s) {
   if (n_photons == 0) return cudaSuccess;
-  unsigned long long blocks = (n_photons + 255) / 256;
-  const unsigned long long maxb = static_cast<unsigned long long>(n_sm) * 8ull;
-  if (blocks > maxb) blocks = maxb;
-  trace_paths_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(M, S, seed, photon0, n_photons, r_reject,
+  trace_paths_kernel<<<trace_grid(n_photons, n_sm), 256, 0, s>>>(M, S, seed, photon0, n_photons, r_reject,
                                                                    max_scatter, max_paths, stride, out_xyz, out_n,
                                                                    count);
   return cudaGetLastError();

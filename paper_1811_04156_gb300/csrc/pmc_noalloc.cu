@@ -28,27 +28,25 @@ struct NoAllocPairs {
   DPair p[kNoAllocMaxPairs];
 };
 
-__global__ void __launch_bounds__(256) trace_pairs_kernel(const DMedium M, const NoAllocPairs pairs,
-                                                          unsigned long long seed, unsigned long long photon0,
-                                                          unsigned long long n_photons, float r_reject,
-                                                          int max_scatter, double* __restrict__ scratch) {
+__global__ void __launch_bounds__(256)
+    trace_pairs_kernel(const DMedium M, const NoAllocPairs pairs, unsigned long long seed, unsigned long long photon0,
+                       unsigned long long n_photons, float r_reject, int max_scatter, double* __restrict__ scratch) {
   __shared__ double sh[8 * 5];
   const DPair& S = pairs.p[blockIdx.y];
   const uint32_t k0 = static_cast<uint32_t>(seed), k1 = static_cast<uint32_t>(seed >> 32);
   double v[5] = {0, 0, 0, 0, 0};
-  const unsigned long long stride = static_cast<unsigned long long>(gridDim.x) * blockDim.x;
-  for (unsigned long long q = blockIdx.x * blockDim.x + threadIdx.x; q < n_photons; q += stride) {
-    const PhotonResult pr = trace_photon<false>(M, S, k0, k1, photon0 + q, r_reject, max_scatter, nullptr, nullptr,
-                                                nullptr);
-    v[3] += 1.0;
-    if (pr.hit) {
-      const double W = static_cast<double>(expf(pr.lw));
-      v[0] += W;
-      v[1] += W * W;
-      v[2] += 1.0;
-      v[4] += W * static_cast<double>(pr.L);
-    }
-  }
+  unsigned int emitted = 0;
+  trace_photons<false>(M, S, k0, k1, photon0, n_photons, r_reject, max_scatter,
+                [&](unsigned long long, const PhotonResult& pr) {
+                  if (++emitted == 0u) v[3] += 4294967296.0;
+                  if (!pr.hit) return;
+                  const double W = static_cast<double>(expf(pr.lw));
+                  v[0] += W;
+                  v[1] += W * W;
+                  v[2] += 1.0;
+                  v[4] += W * static_cast<double>(pr.L);
+                });
+  v[3] += static_cast<double>(emitted);
   const int t = threadIdx.x;
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
