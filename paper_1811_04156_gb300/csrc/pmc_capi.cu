@@ -1583,7 +1583,7 @@ int pmc_logp(pmc_ctx_t ctx, pmc_medium_t med, pmc_geom_t geom, int pair, const f
   if (!ctx || !med || !d || !xyz || !n || !out_logp) return fail(PMC_ERR_INVALID, "bad argument");
   if (batch < 0 || cap < 2 || cap > (1 << 20)) return fail(PMC_ERR_INVALID, "bad batch or cap");
   CK(cudaSetDevice(ctx->device));
-  CK(launch_logp(med->d, *d, xyz, n, batch, cap, out_logp, nullptr, static_cast<cudaStream_t>(stream)));
+  CK(launch_logp(med->d, *d, xyz, n, batch, cap, out_logp, nullptr, ctx->n_sm, static_cast<cudaStream_t>(stream)));
   return PMC_OK;
 }
 
@@ -1593,7 +1593,7 @@ int pmc_logp_grad(pmc_ctx_t ctx, pmc_medium_t med, pmc_geom_t geom, int pair, co
   if (!ctx || !med || !d || !xyz || !n || !out_grad) return fail(PMC_ERR_INVALID, "bad argument");
   if (batch < 0 || cap < 2 || cap > (1 << 20)) return fail(PMC_ERR_INVALID, "bad batch or cap");
   CK(cudaSetDevice(ctx->device));
-  CK(launch_logp(med->d, *d, xyz, n, batch, cap, out_logp, out_grad, static_cast<cudaStream_t>(stream)));
+  CK(launch_logp(med->d, *d, xyz, n, batch, cap, out_logp, out_grad, ctx->n_sm, static_cast<cudaStream_t>(stream)));
   return PMC_OK;
 }
 

@@ -123,7 +123,7 @@ cudaError_t launch_init(const InitParams& p, cudaStream_t s);
 
 // pmc_kernels.cu
 cudaError_t launch_logp(const DMedium& M, const DPair& S, const float* xyz, const int* n, int batch, int cap,
-                        float* out_logp, float* out_grad, cudaStream_t s);
+                        float* out_logp, float* out_grad, int n_sm, cudaStream_t s);
 cudaError_t launch_score(const DMedium& M, const DPair& S, const float* xyz, const int* n, int batch, int cap,
                          float* out, int n_theta, const double* ls, const double* la, cudaStream_t s);
 cudaError_t launch_z2(const DMedium& M, const DPair* pairs, int n_pairs, int n_v, int n_phi, double* out,
