@@ -644,6 +644,8 @@ static ChainParams class_params(pmc_chains_t ch, size_t k, unsigned long long n_
   p.chain_hi = cl.hi;
   p.n_steps = n_steps;
   p.smem_cap = cl.smem_cap;
+  // a chain's results do not depend on the shared window: the cap alone sets the rounding
+  p.birth_fuse_z = cl.max_cap > 256;
   return p;
 }
 

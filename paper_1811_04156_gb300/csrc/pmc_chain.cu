@@ -23,6 +23,12 @@
 // Estimators: observables (n, length L, sum of d log sigma/dg) change only on
 // acceptance, so each state's values are added once with its dwell time into
 // FP32 partials that are flushed into lane-distributed FP64 accumulators.
+// Code size: the general kernels wait for instruction fetch (3 to 4.4 of some
+// 10 stall cycles per issue), since a step's code is longer than the
+// instruction cache serves to warps in different phases.  Loops over a path
+// are therefore kept rolled (`#pragma unroll 1`): 100 layers, 30,720 chains x
+// 500 steps 14.9 -> 13.4 ms; two-sensor tree moves, 4,096 chains x 200 steps
+// 5.3 -> 4.1 ms.
 // kTree adds the paper's within-dimension move in tree coordinates (section
 // "Path proposal distribution"; appendix "Path space coordinate system"): the
 // whole path is re-expressed node by node in recursive bispherical systems,
@@ -32,165 +38,16 @@
 
 #include "pmc_internal.h"
 #include "pmc_tree.cuh"
+#include "pmc_warp.cuh"
 
 namespace pmc {
 
 namespace {
 
-constexpr unsigned kFull = 0xffffffffu;
-constexpr int kRefreshSteps = 256;  // recompute the running sums from the caches
-constexpr int kFlushAccepts = 64;   // FP32 partials -> FP64 accumulators
-constexpr int kRngWords = 8;        // staged words per step
-constexpr int kPairWords = 64;      // shared slot for the pair constants (floats)
-static_assert(sizeof(DPair) <= kPairWords * sizeof(float), "pair slot too small");
-constexpr int kMedWords = 48;       // wavelength sampling: the medium at the chain's wavelength (floats)
-static_assert(sizeof(DMedium) <= kMedWords * sizeof(float), "medium slot too small");
-
-enum Move { MV_INTERIOR = 0, MV_END = 1, MV_BIRTH = 2, MV_DEATH = 3 };
-
-// View of one chain's path: entries [0, S) of every array live in the warp's
-// shared memory, entries [S, cap) in the chain's global block (same layout:
-// array a at offset a * stride).  kTb: tau_b per segment is cached (layered
-// media); otherwise it is b * length.  kGt: d log sigma / dg per vertex is
-// cached (gradients requested).  kSpill = false: the whole cap fits (S >= cap)
-// and every access goes to shared memory.
-template <bool kTb, bool kGt, bool kSpill>
-struct WarpPath {
-  static constexpr int kArrays = 6 + (kTb ? 1 : 0) + (kGt ? 1 : 0);
-  static constexpr int kX = 0, kY = 1, kZ = 2, kSeg = 3, kLen = 4, kVt = 5, kTbA = 6, kGtA = 6 + (kTb ? 1 : 0);
-  float* sm;   // shared arrays, stride S
-  float* gm;   // global block of the chain, stride cap
-  int S, cap;
-  float b;
-  template <int a>
-  __device__ __forceinline__ float ld(int i) const {
-    if (kSpill && i >= S) return gm[a * cap + i];
-    return sm[a * S + i];
-  }
-  template <int a>
-  __device__ __forceinline__ void st(int i, float v) const {
-    if (kSpill && i >= S) gm[a * cap + i] = v;
-    else sm[a * S + i] = v;
-  }
-  __device__ float3 pos(int i) const { return f3(ld<kX>(i), ld<kY>(i), ld<kZ>(i)); }
-  __device__ void set_pos(int i, float3 p) const {
-    st<kX>(i, p.x);
-    st<kY>(i, p.y);
-    st<kZ>(i, p.z);
-  }
-  __device__ float seg(int i) const { return ld<kSeg>(i); }
-  __device__ float len(int i) const { return ld<kLen>(i); }
-  __device__ float vt(int i) const { return ld<kVt>(i); }
-  __device__ void set_seg(int i, float v) const { st<kSeg>(i, v); }
-  __device__ void set_len(int i, float v) const { st<kLen>(i, v); }
-  __device__ void set_vt(int i, float v) const { st<kVt>(i, v); }
-  __device__ float tb(int i) const {
-    if constexpr (kTb) return ld<kTbA>(i);
-    else return b * ld<kLen>(i);
-  }
-  __device__ float gt(int i) const {
-    if constexpr (kGt) return ld<kGtA>(i);
-    else return 0.f;
-  }
-  __device__ void set_tb(int i, float v) const {
-    if constexpr (kTb) st<kTbA>(i, v);
-  }
-  __device__ void set_gt(int i, float v) const {
-    if constexpr (kGt) st<kGtA>(i, v);
-  }
-};
-
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
   return v;
-}
-
-// d log p / d f_v with the terms spread over lanes: lanes 0-1 the two segment
-// factors that end / start at v, lanes 2-4 the scattering angles at v-1, v,
-// v+1, lane 5 the emission and detection factors; a shuffle tree sums them
-// and every lane returns the total.  Same formulas as grad_vertex.
-template <class PosF>
-__device__ float3 grad_vertex_warp(const DMedium& M, const DPair& S, float zoff, PosF pos, int n, int v, int lane) {
-  float3 pv[5];
-#pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    const int k = min(max(v - 2 + i, 0), n - 1);
-    pv[i] = pos(k);
-  }
-  float3 rh[4];
-  float el[4];
-  bool ex[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int k = v - 2 + i;
-    ex[i] = (k >= 0 && k <= n - 2);
-    const float3 r = pv[i + 1] - pv[i];
-    const float rr = dot(r, r);
-    const float ir = ex[i] ? rsqrtf(rr) : 1.0f;
-    el[i] = ex[i] ? rr * ir : 1.0f;
-    rh[i] = ir * r;
-  }
-  float3 g = f3(0.f, 0.f, 0.f);
-  if (lane < 2) {
-    const bool e = (lane == 0) ? ex[1] : ex[2];
-    const float3 P = (lane == 0) ? pv[1] : pv[2];
-    const float3 Q = (lane == 0) ? pv[2] : pv[3];
-    const float3 r = (lane == 0) ? rh[1] : rh[2];
-    const float l = (lane == 0) ? el[1] : el[2];
-    if (e) {
-      float3 dP, dQ;
-      dtau_dends(M, zoff, P, Q, l, r, dP, dQ);
-      g = (lane == 0) ? (f3(0.f, 0.f, 0.f) - dQ - (2.0f / l) * r) : ((2.0f / l) * r - dP);
-    }
-  } else if (lane < 5) {
-    const int k = v - 3 + lane;
-    if (k >= 1 && k <= n - 2) {
-      const float3 A = (lane == 2) ? rh[0] : ((lane == 3) ? rh[1] : rh[2]);
-      const float3 B = (lane == 2) ? rh[1] : ((lane == 3) ? rh[2] : rh[3]);
-      const float lA = (lane == 2) ? el[0] : ((lane == 3) ? el[1] : el[2]);
-      const float lB = (lane == 2) ? el[1] : ((lane == 3) ? el[2] : el[3]);
-      const float alpha = (lane == 2) ? 0.f : ((lane == 3) ? 1.f : -1.f);
-      const float beta = (lane == 2) ? 1.f : ((lane == 3) ? -1.f : 0.f);
-      const float w = phase_dlogdc(M, A, B);
-      g = w * (alpha * drdot(A, lA, B) + beta * drdot(B, lB, A));
-    }
-  } else if (lane == 5) {
-    if (S.emission != 0) {
-      const float3 ed = f3(S.dir[0], S.dir[1], S.dir[2]);
-      if (v == 1) g = g + S.kappa * drdot(rh[1], el[1], ed);
-      if (v == 0 && ex[2]) g = g - S.kappa * drdot(rh[2], el[2], ed);
-    }
-    if (v == n - 2 || v == n - 1) {
-      const float3 e = (v == n - 1) ? pv[2] : pv[3];
-      const float3 rhat = (v == n - 1) ? rh[1] : rh[2];
-      const float ell = (v == n - 1) ? el[1] : el[2];
-      float3 nu = (e - f3(S.c[0], S.c[1], S.c[2])) - f3(S.c_lo[0], S.c_lo[1], S.c_lo[2]);
-      const float dn = sqrtf(dot(nu, nu));
-      nu = (1.0f / dn) * nu;
-      const float u = -dot(rhat, nu);
-      const float3 t1 = drdot(rhat, ell, nu);
-      if (v == n - 2) {
-        g = g + (1.0f / u) * t1;
-      } else {
-        const float3 t2 = drdot(nu, dn, rhat);
-        g = g - (1.0f / u) * (t1 + t2);
-        if (S.rho != 0) {
-          const float3 rh_ = f3(S.rho_hat[0], S.rho_hat[1], S.rho_hat[2]);
-          const float x = dot(nu, rh_);
-          const float dl = 3.0f - 2.0f * tanhf(fmaf(2.0f, x, 0.7f));
-          g = g + dl * drdot(nu, dn, rh_);
-        }
-      }
-    }
-  }
-#pragma unroll
-  for (int o = 1; o < 8; o <<= 1) {
-    g.x += __shfl_xor_sync(kFull, g.x, o);
-    g.y += __shfl_xor_sync(kFull, g.y, o);
-    g.z += __shfl_xor_sync(kFull, g.z, o);
-  }
-  return f3(__shfl_sync(kFull, g.x, 0), __shfl_sync(kFull, g.y, 0), __shfl_sync(kFull, g.z, 0));
 }
 
 struct Sums {
@@ -200,6 +57,7 @@ struct Sums {
 template <class WP>
 __device__ Sums path_sums(const WP& w, int n, int lane) {
   float L = 0.f, G = 0.f;
+#pragma unroll 1
   for (int i = lane; i < n; i += 32) {
     G += w.gt(i);
     if (i <= n - 2) L += w.len(i);
@@ -246,6 +104,7 @@ __device__ __forceinline__ void vs_factors(const DMedium& M, const DPair& S, flo
 template <bool kGen, bool kCall, class WP>
 __device__ float refresh_caches(const DMedium& M, const DPair& S, float zoff, const WP& w, int n, int lane) {
   float lp = 0.f;
+#pragma unroll 1
   for (int i = lane; i < n; i += 32) {
     const float3 P = w.pos(i);
     const float3 Pp = (i >= 1) ? w.pos(i - 1) : P;
@@ -269,6 +128,7 @@ __device__ float refresh_caches(const DMedium& M, const DPair& S, float zoff, co
 // Shift entries [a, e) of the vertex-indexed and segment-indexed arrays.
 template <class WP>
 __device__ void shift_right(const WP& w, int a, int e_vtx, int e_seg, int lane) {
+#pragma unroll 1
   for (int base = e_vtx - 1; base >= a; base -= 32) {
     const int i = base - lane;
     const bool ok = i >= a;
@@ -285,6 +145,7 @@ __device__ void shift_right(const WP& w, int a, int e_vtx, int e_seg, int lane) 
 
 template <class WP>
 __device__ void shift_left(const WP& w, int a, int e_vtx, int e_seg, int lane) {
+#pragma unroll 1
   for (int base = a; base < e_vtx; base += 32) {
     const int i = base + lane;
     const bool ok = i < e_vtx;
@@ -318,6 +179,7 @@ __device__ int select_segment(const WP& w, int nseg, float u, float& total, int 
   const int lo = lane * m;
   const int hi = min(lo + m, nseg);
   float local = 0.f;
+#pragma unroll 1
   for (int i = lo; i < hi; ++i) local += w.tb(i);
   float incl = local;
 #pragma unroll
@@ -334,6 +196,7 @@ __device__ int select_segment(const WP& w, int nseg, float u, float& total, int 
   if (lane == owner) {
     float cum = incl - local;
     k = hi - 1;
+#pragma unroll 1
     for (int i = lo; i < hi; ++i) {
       cum += w.tb(i);
       if (cum > target) { k = i; break; }
@@ -358,6 +221,7 @@ __device__ float tree_propose(const DMedium& M, const DPair& S, float zoff, cons
   auto opos = [&](int i) { return w.pos(i); };
   auto npos = [&](int i) { return f3(nx[i], ny[i], nz[i]); };
   float lj = 0.f;  // log J(x') - log J(x), lane partials
+#pragma unroll 1
   for (int m = 1 + lane; m <= n - 2; m += 32) {
     const float3 zc = tree_step_node(opos, m, n, vref, step, t, static_cast<uint32_t>(c), key0, key1, lj);
     nx[m] = zc.x;
@@ -373,6 +237,7 @@ __device__ float tree_propose(const DMedium& M, const DPair& S, float zoff, cons
   __syncwarp();
   for (int d = 0;; ++d) {
     bool any = false;
+#pragma unroll 1
     for (int j0 = 0; j0 < (1 << d); j0 += 32) {
       const int j = j0 + lane;
       int k = 0, l = 0, kp = -1, lp = -1;
@@ -391,6 +256,7 @@ __device__ float tree_propose(const DMedium& M, const DPair& S, float zoff, cons
   }
   // log p of the new path
   float lp = 0.f;
+#pragma unroll 1
   for (int i = lane; i < n; i += 32) {
     const float3 Pc = npos(i);
     const float3 Pp = (i >= 1) ? npos(i - 1) : Pc;
@@ -414,6 +280,7 @@ __device__ float tree_propose(const DMedium& M, const DPair& S, float zoff, cons
 __device__ __forceinline__ bool hmc_path_valid(const DPair& S, const float* nx, const float* ny, const float* nz,
                                                int n, int lane) {
   bool ok = true;
+#pragma unroll 1
   for (int k = lane; k <= n - 2; k += 32) {
     const float3 P = f3(nx[k], ny[k], nz[k]);
     const float3 Q = f3(nx[k + 1], ny[k + 1], nz[k + 1]);
@@ -431,6 +298,7 @@ __device__ __forceinline__ void hmc_kick(const DMedium& M, const DPair& S, float
                                          float h, int lane) {
   if (!hmc_path_valid(S, nx, ny, nz, n, lane)) return;
   auto npos = [&](int i) { return f3(nx[i], ny[i], nz[i]); };
+#pragma unroll 1
   for (int i = 1 + lane; i <= n - 2; i += 32) {
     const float3 g = grad_vertex(M, S, zoff, npos, n, i);
     mx[i] = fmaf(h, g.x, mx[i]);
@@ -446,6 +314,7 @@ __device__ float hmc_propose(const DMedium& M, const DPair& S, float zoff, const
                              float* nz, float* mx, float* my, float* mz, int n, float eps, int L,
                              unsigned long long t, int c, uint32_t key0, uint32_t key1, int lane) {
   float k0 = 0.f;
+#pragma unroll 1
   for (int i = lane; i < n; i += 32) {
     const float3 P = w.pos(i);
     nx[i] = P.x;
@@ -469,8 +338,10 @@ __device__ float hmc_propose(const DMedium& M, const DPair& S, float zoff, const
   }
   __syncwarp();
   hmc_kick(M, S, zoff, nx, ny, nz, mx, my, mz, n, 0.5f * eps, lane);
+#pragma unroll 1
   for (int st = 1; st <= L; ++st) {
     __syncwarp();
+#pragma unroll 1
     for (int i = 1 + lane; i <= n - 2; i += 32) {
       nx[i] = fmaf(eps, mx[i], nx[i]);
       ny[i] = fmaf(eps, my[i], ny[i]);
@@ -481,6 +352,7 @@ __device__ float hmc_propose(const DMedium& M, const DPair& S, float zoff, const
   }
   __syncwarp();
   float k1 = 0.f, lp = 0.f;
+#pragma unroll 1
   for (int i = lane; i < n; i += 32) {
     if (i >= 1 && i <= n - 2) k1 += mx[i] * mx[i] + my[i] * my[i] + mz[i] * mz[i];
     const float3 Pc = f3(nx[i], ny[i], nz[i]);
@@ -535,11 +407,6 @@ __device__ __forceinline__ void flush64(Accum& a, int lane) {
   a.nflush = 0;
 }
 
-// Pre-transformed random numbers of one step (8 staged words):
-//   lo.x = 23-bit index draw | move type << 24, lo.y = log u (accept),
-//   within: lo.z, lo.w, hi.x = standard normals, hi.y = vMF cosine,
-//           hi.z, hi.w = cos, sin of the vMF azimuth
-//   birth:  lo.z = u for cos s, lo.w = sinh t, hi.x = cosh t, hi.y, hi.z = cos, sin of phi
 // Launch bounds: the general tree-move kernel takes up to 128 registers (4
 // CTAs of 128 threads per SM), which holds its out-of-line density call
 // without spills (+2 % on the two-sensor scene); the general Cartesian
@@ -587,6 +454,7 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
     {
       const int* src = reinterpret_cast<const int*>(P.pairs + P.chain_pair[c]);
       int* dst = reinterpret_cast<int*>(spair);
+#pragma unroll 1
       for (int q = lane; q < static_cast<int>(sizeof(DPair) / sizeof(int)); q += 32) dst[q] = src[q];
       __syncwarp();
     }
@@ -612,6 +480,7 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
       __syncwarp();
     }
     // the shared window holds entries [0, min(n, S)); the rest stays in the global block
+#pragma unroll 1
     for (int i = lane; i < min(n, cap_s); i += 32) {
       w.sm[WP::kX * cap_s + i] = gx[i];
       w.sm[WP::kY * cap_s + i] = gy[i];
@@ -645,34 +514,8 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
       // ---- lane-parallel random numbers of steps step0+s0 .. +31 ----
       {
         const unsigned long long tl = step0 + s0 + lane;
-        const uint4 ra = philox4x32_10(make_uint4(static_cast<uint32_t>(tl), static_cast<uint32_t>(tl >> 32),
-                                                  static_cast<uint32_t>(c) + P.chain_id0, PUR_STEP_A), key0, key1);
-        const uint4 rb = philox4x32_10(make_uint4(static_cast<uint32_t>(tl), static_cast<uint32_t>(tl >> 32),
-                                                  static_cast<uint32_t>(c) + P.chain_id0, PUR_STEP_B), key0, key1);
-        const uint32_t um = ra.x >> 9;
-        const uint32_t type = um < R.thr_within ? 0u : (um < R.thr_birth ? 2u : 3u);
-        uint4 lo = make_uint4((ra.y >> 9) | (type << 24), __float_as_uint(__logf(u01(ra.z))), 0u, 0u);
-        uint4 hi;
-        const float ub0 = u01(rb.x), ub1 = u01(rb.y), ub2 = u01(rb.z), ub3 = u01(rb.w);
-        if (type == 0u) {
-          float s1, c1, s2, c2;
-          const float r1 = m_sqrt<true>(-2.0f * __logf(ub0));
-          sincospif(2.0f * ub1, &s1, &c1);
-          const float r2 = m_sqrt<true>(-2.0f * __logf(ub2));
-          sincospif(2.0f * ub3, &s2, &c2);
-          lo.z = __float_as_uint(r1 * c1);
-          lo.w = __float_as_uint(r1 * s1);
-          const float wv = 1.0f + __fdividef(__logf(fmaf(1.0f - ub0, S.exp_m2ke, ub0)), S.kappa_end);
-          hi = make_uint4(__float_as_uint(r2 * c2), __float_as_uint(wv), __float_as_uint(c1), __float_as_uint(s1));
-        } else {
-          const float et = __fdividef(ub1, 1.0f - ub1);
-          const float iet = __fdividef(1.0f - ub1, ub1);
-          float s3, c3;
-          sincospif(2.0f * ub2, &s3, &c3);
-          lo.z = __float_as_uint(ub0);
-          lo.w = __float_as_uint(0.5f * (et - iet));
-          hi = make_uint4(__float_as_uint(0.5f * (et + iet)), __float_as_uint(c3), __float_as_uint(s3), 0u);
-        }
+        uint4 lo, hi;
+        const uint32_t type = stage_step(R, S, tl, static_cast<uint32_t>(c) + P.chain_id0, key0, key1, lo, hi);
         __syncwarp();
         rng[2 * lane] = lo;
         rng[2 * lane + 1] = hi;
@@ -685,6 +528,7 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
         A.prop_d += __popc(__ballot_sync(kFull, live && type == 3u));
       }
       const int cnt = static_cast<int>(min(32ull, P.n_steps - s0));
+#pragma unroll 1
       for (int i = 0; i < cnt; ++i) {
         const uint4 lo = rng[2 * i];
         const uint4 hi = rng[2 * i + 1];
@@ -707,11 +551,13 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
             const float gain = hmc_propose<kGen>(M, S, zoff, w, tnx, tny, tnz, hmx, hmy, hmz, n, R.mala_eps,
                                                  R.hmc_steps, t, cid, key0, key1, lane);
             float lpo = 0.f;
+#pragma unroll 1
             for (int q = lane; q < n; q += 32) lpo += w.vt(q) + ((q <= n - 2) ? w.seg(q) : 0.f);
             lpo = warp_sum(lpo);
             if (logu < gain - lpo) {
               A.acc_i++;
               close_state(A, t, R.burn_in, n, L, G);
+#pragma unroll 1
               for (int q = lane; q < n; q += 32) w.set_pos(q, f3(tnx[q], tny[q], tnz[q]));
               __syncwarp();
               refresh_caches<kGen, kGen && kTree>(M, S, zoff, w, n, lane);
@@ -739,11 +585,13 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
             const float gain = tree_propose<kGen>(M, S, zoff, w, tnx, tny, tnz, n, end, step, vref, t, cid, key0, key1,
                                                   lane);
             float lpo = 0.f;
+#pragma unroll 1
             for (int q = lane; q < n; q += 32) lpo += w.vt(q) + ((q <= n - 2) ? w.seg(q) : 0.f);
             lpo = warp_sum(lpo);
             if (logu < gain - lpo) {
               A.acc_i++;
               close_state(A, t, R.burn_in, n, L, G);
+#pragma unroll 1
               for (int q = lane; q < n; q += 32) w.set_pos(q, f3(tnx[q], tny[q], tnz[q]));
               __syncwarp();
               refresh_caches<kGen, kGen && kTree>(M, S, zoff, w, n, lane);
@@ -809,7 +657,7 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
             const float3 z = f3(__uint_as_float(lo.z), __uint_as_float(lo.w), __uint_as_float(hi.x));
             if constexpr (kGen && kX == 0) {
               if (R.within == 1) {
-                gx_mala = grad_vertex_warp(M, S, zoff, [&](int k) { return w.pos(k); }, n, j, lane);
+                gx_mala = grad_vertex_warp<32>(M, S, zoff, [&](int k) { return w.pos(k); }, n, j, lane);
                 const float h = 0.5f * R.mala_eps * R.mala_eps;
                 fnew = fj + h * gx_mala + R.mala_eps * z;
               } else {
@@ -843,8 +691,9 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
             cs = fminf(fmaxf(cs, -1.0f), 1.0f);
             const float sn = m_sqrt<true>(fmaxf(0.f, (1.0f - cs) * (1.0f + cs)));
             const float sc = __fdividef(gamma, __uint_as_float(hi.x) - cs);
-            fnew = 0.5f * (Af + Bf) +
-                   sc * (__uint_as_float(lo.w) * rh + sn * (__uint_as_float(hi.y) * xi + __uint_as_float(hi.z) * ze));
+            fnew = birth_point<kGen>(
+                Af, Bf, sc, __uint_as_float(lo.w) * rh + sn * (__uint_as_float(hi.y) * xi + __uint_as_float(hi.z) * ze),
+                P.birth_fuse_z);
             const float tbk = w.tb(k);
             extra = R.log_pd - __logf(static_cast<float>(n - 1)) - R.log_pb - __logf(__fdividef(tbk, total)) -
                     log_insert_density<true>(M, R, zoff, Af, Bf, fnew);
@@ -915,6 +764,7 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
             // T_b of the reduced path, summed afresh so that decisions depend
             // only on the current state (split runs replay exactly)
             float part = 0.f;
+#pragma unroll 1
             for (int q = lane; q < n - 1; q += 32) part += w.tb(q);
             const float tb_new = __shfl_sync(kFull, ntb, 0);
             const float Tb_red = warp_sum(part) + dtb;
@@ -923,7 +773,7 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
           }
           if constexpr (kGen && kX == 0) {
             if (move == MV_INTERIOR && R.within == 1 && isfinite(dlp)) {
-              const float3 gy = grad_vertex_warp(M, S, zoff, newpos, n, jj, lane);
+              const float3 gy = grad_vertex_warp<32>(M, S, zoff, newpos, n, jj, lane);
               const float h = 0.5f * R.mala_eps * R.mala_eps;
               const float3 fj = w.pos(jj);
               const float3 dfw = fnew - fj - h * gx_mala;
@@ -998,6 +848,7 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
     if (lane == ACC_ACC + 3) extra_w = static_cast<double>(A.acc_d);
     A.my += extra_w;
     if (lane < ACC_WORDS) P.acc[static_cast<size_t>(c) * ACC_WORDS + lane] = A.my;
+#pragma unroll 1
     for (int i = lane; i < min(n, cap_s); i += 32) {
       gx[i] = w.sm[WP::kX * cap_s + i];
       gy[i] = w.sm[WP::kY * cap_s + i];
@@ -1036,6 +887,7 @@ __global__ void init_kernel(const InitParams p) {
       p.status[c] = ST_BAD_N;
       n = 2;
     }
+#pragma unroll 1
     for (int i = 0; i < n; ++i) {
       gx[i] = ux[i] - S.org[0];
       gy[i] = ux[st + i] - S.org[1];
@@ -1051,6 +903,7 @@ __global__ void init_kernel(const InitParams p) {
     const uint32_t k0 = static_cast<uint32_t>(p.R.seed), k1 = static_cast<uint32_t>(p.R.seed >> 32);
     gx[0] = gy[0] = gz[0] = 0.f;
     const int kk = n - 2;
+#pragma unroll 1
     for (int i = 1; i <= kk; ++i) {
       const float fr = static_cast<float>(i) / static_cast<float>(kk + 1);
       const uint4 r = philox4x32_10(make_uint4(static_cast<uint32_t>(i), 0u, static_cast<uint32_t>(c) + p.chain_id0, PUR_INIT),
@@ -1070,6 +923,7 @@ __global__ void init_kernel(const InitParams p) {
   }
   p.n[c] = n;
   p.step[c] = 0ull;
+#pragma unroll 1
   for (int k = 0; k < ACC_WORDS; ++k) p.acc[static_cast<size_t>(c) * ACC_WORDS + k] = 0.0;
 }
 

@@ -192,6 +192,7 @@ __device__ __forceinline__ void seg_tau(const DMedium& M, float zP, float zQ, fl
   const int l0 = min(lP, lQ), l1 = max(lP, lQ);
   const float inv_span = 1.0f / (zhi - zlo);
   float sa = 0.0f, sb = 0.0f;
+#pragma unroll 1
   for (int l = l0; l <= l1; ++l) {
     const float lo = (l == l0) ? zlo : M.z0 + l * M.dz;
     const float hi = (l == l1) ? zhi : M.z0 + (l + 1) * M.dz;
@@ -486,6 +487,7 @@ __device__ inline float spectrum_log(const DRun& R, float lam) {
 __device__ inline float spectrum_quantile(const DRun& R, float u) {
   const int K = R.n_spec;
   float t = u;
+#pragma unroll 1
   for (int i = 0; i + 1 < K; ++i) {
     const float h = R.spec_x[i + 1] - R.spec_x[i];
     const float y0 = R.spec_y[i], y1 = R.spec_y[i + 1];

@@ -59,6 +59,7 @@ struct ChainParams {
   int chain_lo, chain_hi;       // chains [lo, hi) of this launch
   unsigned long long n_steps;
   int smem_cap;                 // vertex capacity of one warp's shared arrays
+  int birth_fuse_z;             // rounding of a birth's z (birth_point)
 };
 
 // Kernel launchers (pmc_chain.cu)

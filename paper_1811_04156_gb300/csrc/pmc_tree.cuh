@@ -32,6 +32,7 @@ __device__ __forceinline__ bool tree_interval(int n, int d, int j, int& k, int& 
   k = 0;
   l = n - 1;
   kp = lp = -1;
+#pragma unroll 1
   for (int b = d - 1; b >= 0; --b) {
     if (l - k < 2) return false;
     const int mid = (k + l) >> 1;
