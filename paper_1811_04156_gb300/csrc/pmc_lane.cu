@@ -18,12 +18,18 @@
 // is a path length index the shared window directly.
 //
 // Layout: the first W vertices of each chain (W = smem_cap) live in the
-// warp's shared block as [array][vertex][lane] floats, so that every lane
-// stays in its own bank whatever vertex it touches; entries W..cap-1 live in
-// the chain's global block (array a at a * cap), as in the warp kernel's
-// spill mode.  Tree moves add three arrays for the proposed path.  Positions are read from and written back to the global block
-// at the start and end of a residency; the cached factors are rebuilt at the
-// start.
+// warp's shared block (LanePath below), entries W..cap-1 in the chain's global
+// block (array a at a * cap), as in the warp kernel's spill mode.  Tree moves
+// add three arrays for the proposed path.  Positions are read from and written
+// back to the global block at the start and end of a residency; the cached
+// factors are rebuilt at the start.
+//
+// Bound by instruction issue (64 % of the slots with 3.4 warps per scheduler).
+// The float4 / float2 layout and the branch-free factors took the detector run
+// (65,536 chains, mean n 11) from 47.7 to 43.6 warp instructions per proposal:
+// 4,000 steps with the estimate 18.6 -> 16.1 ms (float arrays and branching
+// factors -> branch-free 17.4 -> vectors 16.1); the MALA gradients run 17.5 ->
+// 16.9 ms.
 #include "pmc_internal.h"
 #include "pmc_tree.cuh"
 
@@ -41,28 +47,83 @@ constexpr int kFlush = 64;           // FP32 partials -> FP64 accumulators
 enum { AX = 0, AY = 1, AZ = 2, ASEG = 3, ALEN = 4, AVT = 5, AGT = 6 };
 enum Move { MV_INTERIOR = 0, MV_END = 1, MV_BIRTH = 2, MV_DEATH = 3 };
 
-// kRow: floats per vertex row of the warp's shared block (32, one per lane;
-// 33 for tree moves, so that lanes working on vertices of one chain in the
-// warp's pooled passes fall into different banks)
+// One chain's path.  Gaussian and MALA moves (kVec): a vertex's position and
+// factor are one float4 and its segment's factor and length one float2, so
+// that a vertex moves with two shared accesses instead of six and a vertex
+// read brings its factor along: [vertex][lane] float4, then [vertex][lane]
+// float2 (then d log sigma / dg, [vertex][lane] floats); a warp's 32 lanes read
+// consecutive 16- or 8-byte words whatever vertex each of them touches.  Tree
+// moves: [array][vertex][kRow] floats (33 per row, so that lanes working on
+// vertices of one chain in the warp's pooled passes fall into different banks).
+// Entries from W on live in the chain's global block, array a at a * cap.
 template <int kRow>
 struct LanePath {
-  float* sm;  // this lane's column of the warp's shared block
+  static constexpr bool kVec = kRow == 32;
+  float* sm;  // tree moves: this lane's column; else the warp's block
   float* gm;  // the chain's global block
-  int W, cap;
-  __device__ __forceinline__ float ld(int a, int i) const {
-    return (i < W) ? sm[(a * W + i) * kRow] : gm[a * cap + i];
+  int W, cap, lane;
+  __device__ __forceinline__ float4* va(int i) const { return reinterpret_cast<float4*>(sm) + i * 32 + lane; }
+  __device__ __forceinline__ float2* vb(int i) const { return reinterpret_cast<float2*>(sm + 128 * W) + i * 32 + lane; }
+  __device__ __forceinline__ float* at(int a, int i) const {
+    if constexpr (kVec) {
+      if (a <= AZ) return reinterpret_cast<float*>(va(i)) + a;
+      if (a == AVT) return reinterpret_cast<float*>(va(i)) + 3;
+      if (a == ASEG || a == ALEN) return reinterpret_cast<float*>(vb(i)) + (a - ASEG);
+      return sm + 192 * W + i * 32 + lane;
+    } else {
+      return sm + (a * W + i) * kRow;
+    }
   }
+  __device__ __forceinline__ float ld(int a, int i) const { return (i < W) ? *at(a, i) : gm[a * cap + i]; }
   __device__ __forceinline__ void st(int a, int i, float v) const {
-    if (i < W) sm[(a * W + i) * kRow] = v;
+    if (i < W) *at(a, i) = v;
     else gm[a * cap + i] = v;
   }
-  // entry i of every array in shared memory (i < W): array a at [a * W * kRow]
-  __device__ __forceinline__ float* row(int i) const { return sm + i * kRow; }
-  __device__ __forceinline__ float3 pos(int i) const { return f3(ld(AX, i), ld(AY, i), ld(AZ, i)); }
+  __device__ __forceinline__ float3 pos(int i) const {
+    const float4 v = vertex(i);
+    return f3(v.x, v.y, v.z);
+  }
   __device__ __forceinline__ void set_pos(int i, float3 p) const {
     st(AX, i, p.x);
     st(AY, i, p.y);
     st(AZ, i, p.z);
+  }
+  // position and vertex factor; segment factor and length
+  __device__ __forceinline__ float4 vertex(int i) const {
+    if constexpr (kVec) {
+      if (i < W) return *va(i);
+      return make_float4(gm[AX * cap + i], gm[AY * cap + i], gm[AZ * cap + i], gm[AVT * cap + i]);
+    } else {
+      return make_float4(ld(AX, i), ld(AY, i), ld(AZ, i), ld(AVT, i));
+    }
+  }
+  __device__ __forceinline__ float2 segment(int i) const {
+    if constexpr (kVec) {
+      if (i < W) return *vb(i);
+      return make_float2(gm[ASEG * cap + i], gm[ALEN * cap + i]);
+    } else {
+      return make_float2(ld(ASEG, i), ld(ALEN, i));
+    }
+  }
+  __device__ __forceinline__ void set_vertex(int i, float4 v) const {
+    if constexpr (kVec) {
+      if (i < W) {
+        *va(i) = v;
+        return;
+      }
+    }
+    set_pos(i, f3(v.x, v.y, v.z));
+    st(AVT, i, v.w);
+  }
+  __device__ __forceinline__ void set_segment(int i, float2 v) const {
+    if constexpr (kVec) {
+      if (i < W) {
+        *vb(i) = v;
+        return;
+      }
+    }
+    st(ASEG, i, v.x);
+    st(ALEN, i, v.y);
   }
 };
 
@@ -201,7 +262,7 @@ __device__ float pooled_tree_gain(const ChainParams& P, TreeSlot* slots, float* 
   // every interior node's stepped coordinates, and -log of its volume element at x
   pooled_for(slots, mine ? n_mine - 2 : 0, [&](int src, int idx) {
     const TreeSlot& T = slots[src];
-    const LanePath<kRow> o{cols + src, T.gm, W, T.cap};
+    const LanePath<kRow> o{cols + src, T.gm, W, T.cap, src};
     const Proposal q = proposal_of<kGrad>(T, pool);
     const int m = idx + 1;
     float lj = 0.f;
@@ -255,7 +316,7 @@ __device__ void pooled_tree_commit(const ChainParams& P, TreeSlot* slots, float*
   const int lane = threadIdx.x & 31;
   pooled_for(slots, taken ? slots[lane].n : 0, [&](int src, int i) {
     const TreeSlot& T = slots[src];
-    const LanePath<kRow> o{cols + src, T.gm, W, T.cap};
+    const LanePath<kRow> o{cols + src, T.gm, W, T.cap, src};
     const Proposal q = proposal_of<kGrad>(T, pool);
     const DPair& S = P.pairs[T.pair];
     const int n = T.n;
@@ -286,6 +347,49 @@ __device__ __forceinline__ void lane_refresh_sums(const LanePath<kRow>& w, int n
     for (int q = 0; q < n; ++q) Gs += w.ld(AGT, q);
     G = Gs;
   }
+}
+
+// Entry wlo + i (i = -1 .. 3) of a window of five positions.
+__device__ __forceinline__ float3 lane_window(float3 a, float3 b, float3 c, float3 d, float3 e, int i) {
+  return i < 1 ? (i < 0 ? a : b) : (i < 2 ? c : (i < 3 ? d : e));
+}
+
+// A segment of the proposed path: squared length, its inverse root, direction.
+struct LaneSegment {
+  float3 r, u;
+  float bb, ib;
+};
+__device__ __forceinline__ LaneSegment lane_segment(float3 r) {
+  LaneSegment s;
+  s.r = r;
+  s.bb = dot(r, r);
+  s.ib = rsqrtf(s.bb);
+  s.u = f3(__fmul_rn(s.ib, r.x), __fmul_rn(s.ib, r.y), __fmul_rn(s.ib, r.z));
+  return s;
+}
+
+// log b + log of the phase density between two segments, and d log sigma / dg
+// (phase_term<true, false>).  kFuse: the difference of the directions takes
+// the second one's scaling and the subtraction as one rounding.
+template <bool kFuse>
+__device__ __forceinline__ float lane_phase(const DMedium& M, const LaneSegment& a, const LaneSegment& b, float& gterm) {
+  const float3 dm = kFuse ? f3(__fmaf_rn(-b.ib, b.r.x, a.u.x), __fmaf_rn(-b.ib, b.r.y, a.u.y),
+                               __fmaf_rn(-b.ib, b.r.z, a.u.z))
+                          : f3(__fadd_rn(a.u.x, -b.u.x), __fadd_rn(a.u.y, -b.u.y), __fadd_rn(a.u.z, -b.u.z));
+  const float omc = 0.5f * dot(dm, dm);
+  const float den = fmaf(M.two_g, omc, M.omg2);
+  gterm = M.hg_dg0 - 3.0f * m_div<true>(M.g - 1.0f + omc, den);
+  return M.log_b + fmaf(-1.5f, m_log<true>(den), M.hg_lognorm);
+}
+
+// Factor of the segment that starts at P (non_final: it may not touch the sensor).
+__device__ __forceinline__ float lane_segment_factor(const DMedium& M, const DPair& S, float3 P, const LaneSegment& s,
+                                                     float ell, bool non_final) {
+  const float ta = M.a * ell, tbv = M.b * ell;
+  float seg = -(ta + tbv) - m_log<true>(s.bb);
+  const bool hit = hits_ball<true>(S, P, s.r);
+  if (!(s.bb > 0.0f) || (non_final && hit)) seg = kNegInf;
+  return seg;
 }
 
 // Every step of one chain's residency, on one lane.  Mirrors the warp
@@ -320,15 +424,12 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
     n = 2;
   }
   LanePath<kRow> w;
-  w.sm = col;
+  w.sm = kTree ? col : col - lane;
   w.gm = P.xyz + P.chain_base[c];
   w.W = W;
   w.cap = cap;
-  for (int i = 0; i < min(n, W); ++i) {
-    w.sm[(AX * W + i) * kRow] = w.gm[AX * cap + i];
-    w.sm[(AY * W + i) * kRow] = w.gm[AY * cap + i];
-    w.sm[(AZ * W + i) * kRow] = w.gm[AZ * cap + i];
-  }
+  w.lane = lane;
+  for (int i = 0; i < min(n, W); ++i) w.set_pos(i, f3(w.gm[AX * cap + i], w.gm[AY * cap + i], w.gm[AZ * cap + i]));
   // cached factors of the whole path, with a sliding window of positions
   float lp0 = 0.f, L = 0.f, G = 0.f;
   {
@@ -464,11 +565,10 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
         if (born) {
           float cum = 0.f;
           int below = 0;
-          const float* pl = w.sm + ALEN * W * kRow;
           const int m = min(n - 1, W);
 #pragma unroll 4
           for (int q = 0; q < m; ++q) {
-            cum += M.b * pl[q * kRow];
+            cum += M.b * *w.at(ALEN, q);
             below += (cum <= target) ? 1 : 0;
           }
           for (int q = W; q < n - 1; ++q) {
@@ -485,10 +585,12 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
         // death, IA and IB the segment ends of a birth or about a death
         const int wlo = end ? n - 2 : (within ? jw - 1 : (birth ? k : jd - 1));
         const float3 Q0 = w.pos(max(wlo - 1, 0));
-        const float3 IA = w.pos(wlo);
-        const float3 V = w.pos(min(wlo + 1, n - 1));
-        const float3 IB = w.pos(min(birth ? wlo + 1 : wlo + 2, n - 1));
+        const float4 IA4 = w.vertex(wlo);
+        const float4 V4 = w.vertex(min(wlo + 1, n - 1));
+        const float4 IB4 = w.vertex(min(birth ? wlo + 1 : wlo + 2, n - 1));
         const float3 Y = w.pos(min(birth ? wlo + 2 : wlo + 3, n - 1));
+        const float3 IA = f3(IA4.x, IA4.y, IA4.z), V = f3(V4.x, V4.y, V4.z), IB = f3(IB4.x, IB4.y, IB4.z);
+        const float2 SA = w.segment(wlo), SB = w.segment(min(wlo + 1, n - 1));
         float3 fin = f3(0.f, 0.f, 0.f), fend = f3(0.f, 0.f, 0.f);
         float3 gx = f3(0.f, 0.f, 0.f);  // MALA: d log p / d f_j at the current path
         if constexpr (!kTree) {
@@ -506,7 +608,7 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
           const float3 z = f3(r1 * c1, r1 * s1, r2 * cB);
           if constexpr (kMala) {
             // Langevin step: drift along the local gradient of log p
-            if (within && !end) gx = grad_vertex(M, S, S.zoff, [&](int q) { return w.pos(q); }, n, jw);
+            if (within && !end) gx = grad_vertex(M, S, S.zoff, [&](int q) { return lane_window(Q0, IA, V, IB, Y, q - wlo); }, n, jw);
             const float h = 0.5f * R.mala_eps * R.mala_eps;
             fin = V + h * gx + R.mala_eps * z;
           } else {
@@ -533,7 +635,7 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
           const float sht = 0.5f * (et - iet), cht = 0.5f * (et + iet);
           const float sc = __fdividef(gamma, cht - cs);
           fbirth = 0.5f * (IA + IB) + sc * (sht * rh + sn * (cB * xi + sB * ze));
-          const float tbk = M.b * w.ld(ALEN, k);
+          const float tbk = M.b * SA.y;  // (births: k = wlo)
           extra_b = R.log_pd - __logf(static_cast<float>(n - 1)) - R.log_pb - __logf(__fdividef(tbk, total));
         }
         // the drawn kind's proposal
@@ -546,7 +648,6 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
         const int jj = within ? jw : jd, kk = k;
         const int n_new = birth ? n + 1 : (death ? n - 1 : n);
         const int inew = within ? jw : (birth ? k + 1 : -1);
-        const int olo = wlo;
         const int nc = (end || death) ? 2 : 3;
         const int onc = (end || birth) ? 2 : 3;
         const float3 fnew = within ? (end ? fend : fin) : (birth ? fbirth : f3(0.f, 0.f, 0.f));
@@ -555,77 +656,82 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
         // the insertion density at a birth's or a death's segment ends and vertex
         const float lid = log_insert_density<true>(M, R, S.zoff, IA, IB, IF);
 
-        bool accept = false;
-        float nvt[3] = {0.f, 0.f, 0.f}, nseg[2] = {0.f, 0.f}, nlen[2] = {0.f, 0.f}, ngt[3] = {0.f, 0.f, 0.f};
-        float dlen = 0.f, dG = 0.f;
-        if (proposed) {
-          // new-path positions wlo-1 .. wlo+nc: the current path's entries, a
-          // death's shifted down by one past the removed vertex, the new vertex
-          // at wlo+1 (a birth's entries past it shifted up by one)
-          const float3 Q[5] = {Q0, IA, death ? IB : fnew, death ? Y : IB,
-                               (death || end) ? f3(0.f, 0.f, 0.f) : Y};
-          // the changed vertex and segment factors against the cached ones; the
-          // three per-slot differences are summed as the warp kernel's two
-          // shuffle rounds sum them, (d0 + d1) + d2
-          float d[3], e[3], f[3], gd[3];
-#pragma unroll
-          for (int v = 0; v < 3; ++v) {
-            float nv = 0.f, ns = 0.f, ntb = 0.f, nl = 0.f, ng = 0.f;
-            if (v < nc) {
-              float seg_, tb_, len_;
-              vertex_and_segment<false>(M, S, S.zoff, Q[v], Q[v + 1], Q[v + 2], wlo + v, n_new, nv, ng, seg_, tb_,
-                                        len_);
-              if (v < nc - 1) {
-                ns = seg_;
-                ntb = tb_;
-                nl = len_;
-              }
-            }
-            float ov = 0.f, os = 0.f, otb = 0.f, ol = 0.f, og = 0.f;
-            if (v < onc) {
-              const int o = olo + v;
-              ov = w.ld(AVT, o);
-              if constexpr (kGrad) og = w.ld(AGT, o);
-              if (v < onc - 1) {
-                os = w.ld(ASEG, o);
-                ol = w.ld(ALEN, o);
-                otb = M.b * ol;
-              }
-            }
-            nvt[v] = nv;
-            ngt[v] = ng;
-            if (v < 2) {
-              nseg[v] = ns;
-              nlen[v] = nl;
-            }
-            d[v] = (nv + ns) - (ov + os);
-            e[v] = ntb - otb;
-            f[v] = nl - ol;
-            gd[v] = ng - og;
-          }
-          const float dlp = (d[0] + d[1]) + d[2];
-          dlen = (f[0] + f[1]) + f[2];
-          if constexpr (kGrad) dG = (gd[0] + gd[1]) + gd[2];
-          // a death's T_b of the reduced path, from the current one; one
-          // insertion density for births and deaths: a birth divides by it, a
-          // death multiplies
-          const float dtb = (e[0] + e[1]) + e[2];
-          const float Tb_red = Tb + dtb;
-          const float tb_new = M.b * nlen[0];
-          const float extra_d =
-              -R.log_pd + __logf(static_cast<float>(n - 2)) + R.log_pb + __logf(__fdividef(tb_new, Tb_red));
-          extra = birth ? extra - lid : (death ? extra_d + lid : extra);
-          if (kMala && move == MV_INTERIOR && isfinite(dlp)) {
-            // MALA Hastings ratio q(x | y) / q(y | x), with the gradient at the proposal
-            const float3 gy = grad_vertex(M, S, S.zoff, [&](int k) { return k == jj ? fnew : w.pos(k); }, n, jj);
-            const float h = 0.5f * R.mala_eps * R.mala_eps;
-            const float3 fj = w.pos(jj);
-            const float3 dfw = fnew - fj - h * gx;
-            const float3 dbw = fj - fnew - h * gy;
-            extra = (dot(dfw, dfw) - dot(dbw, dbw)) / (2.0f * R.mala_eps * R.mala_eps);
-          }
-          accept = logu < dlp + extra;
+        // new-path positions wlo-1 .. wlo+nc: the current path's entries, a
+        // death's shifted down by one past the removed vertex, the new vertex
+        // at wlo+1 (a birth's entries past it shifted up by one)
+        const float3 Q2 = death ? IB : fnew, Q3 = death ? Y : IB;
+        const float3 Q4 = (death || end) ? f3(0.f, 0.f, 0.f) : Y;
+        // the changed vertex and segment factors (as vertex_and_segment gives
+        // them) without branches: the four segments about the changed vertices
+        // once, the phase function at each of the three slots, the detection
+        // factor once (the end vertex is slot 1 or 2, the source slot 0).  With
+        // three calls of the branching function, every warp ran each call's
+        // source, end and scattering branches in turn.
+        const LaneSegment g0 = lane_segment(IA - Q0), g1 = lane_segment(Q2 - IA), g2 = lane_segment(Q3 - Q2),
+                          g3 = lane_segment(Q4 - Q3);
+        const bool three = nc == 3;
+        const bool last1 = wlo + 1 == n_new - 1, last2 = three && wlo + 2 == n_new - 1;
+        float nvt[3], ngt[3] = {0.f, 0.f, 0.f}, nseg[2], nlen[2];
+        {
+          float g;
+          const float v0 = lane_phase<false>(M, g0, g1, g);
+          nvt[0] = wlo == 0 ? -kLog4Pi : v0;
+          if constexpr (kGrad) ngt[0] = wlo == 0 ? 0.f : g;
+          const float v1 = lane_phase<false>(M, g1, g2, g);
+          if constexpr (kGrad) ngt[1] = last1 ? 0.f : g;
+          const float v2 = lane_phase<true>(M, g2, g3, g);
+          if constexpr (kGrad) ngt[2] = (last2 || !three) ? 0.f : g;
+          const float det = sensor_term<true>(S, last1 ? g1.u : g2.u, last1 ? Q2 : Q3);
+          nvt[1] = last1 ? det : v1;
+          nvt[2] = three ? (last2 ? det : v2) : 0.f;
         }
+        nlen[0] = g1.bb * g1.ib;
+        nseg[0] = lane_segment_factor(M, S, IA, g1, nlen[0], wlo <= n_new - 3);
+        nlen[1] = three ? g2.bb * g2.ib : 0.f;
+        nseg[1] = lane_segment_factor(M, S, Q2, g2, nlen[1], wlo + 1 <= n_new - 3);
+        if (!three) nseg[1] = 0.f;
+        // ... against the cached ones; the three per-slot differences are
+        // summed as the warp kernel's two shuffle rounds sum them, (d0 + d1) + d2
+        float d[3], e[3], f[3], gd[3];
+#pragma unroll
+        for (int v = 0; v < 3; ++v) {
+          float ov = 0.f, os = 0.f, otb = 0.f, ol = 0.f, og = 0.f;
+          if (v < onc) {
+            ov = v == 0 ? IA4.w : (v == 1 ? V4.w : IB4.w);
+            if constexpr (kGrad) og = proposed ? w.ld(AGT, wlo + v) : 0.f;
+            if (v < onc - 1) {
+              os = v == 0 ? SA.x : SB.x;
+              ol = v == 0 ? SA.y : SB.y;
+              otb = M.b * ol;
+            }
+          }
+          const float ns = v < 2 ? nseg[v] : 0.f, nl = v < 2 ? nlen[v] : 0.f;
+          d[v] = (nvt[v] + ns) - (ov + os);
+          e[v] = (v < 2 ? M.b * nl : 0.f) - otb;
+          f[v] = nl - ol;
+          gd[v] = ngt[v] - og;
+        }
+        const float dlp = (d[0] + d[1]) + d[2];
+        const float dlen = (f[0] + f[1]) + f[2];
+        const float dG = kGrad ? (gd[0] + gd[1]) + gd[2] : 0.f;
+        // a death's T_b of the reduced path, from the current one; one
+        // insertion density for births and deaths: a birth divides by it, a
+        // death multiplies
+        const float dtb = (e[0] + e[1]) + e[2];
+        const float Tb_red = Tb + dtb;
+        const float tb_new = M.b * nlen[0];
+        const float extra_d =
+            -R.log_pd + __logf(static_cast<float>(n - 2)) + R.log_pb + __logf(__fdividef(tb_new, Tb_red));
+        extra = birth ? extra - lid : (death ? extra_d + lid : extra);
+        if (kMala && move == MV_INTERIOR && isfinite(dlp)) {
+          // MALA Hastings ratio q(x | y) / q(y | x), with the gradient at the proposal
+          const float3 gy = grad_vertex(M, S, S.zoff, [&](int q) { return lane_window(Q0, IA, fnew, IB, Y, q - wlo); }, n, jj);
+          const float h = 0.5f * R.mala_eps * R.mala_eps;
+          const float3 dfw = fnew - V - h * gx;
+          const float3 dbw = V - fnew - h * gy;
+          extra = (dot(dfw, dfw) - dot(dbw, dbw)) / (2.0f * R.mala_eps * R.mala_eps);
+        }
+        const bool accept = proposed && logu < dlp + extra;
         if (accept) {
           A.acc_i += (move == MV_INTERIOR);
           A.acc_e += (move == MV_END);
@@ -641,25 +747,52 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
             const bool up = move == MV_BIRTH;
             const int a0 = up ? kk + 1 : jj + 1;
             auto move_any = [&](int i, int j) {
-              w.set_pos(j, w.pos(i));
-              w.st(AVT, j, w.ld(AVT, i));
+              w.set_vertex(j, w.vertex(i));
               if constexpr (kGrad) w.st(AGT, j, w.ld(AGT, i));
-              if (i < n - 1) {
-                w.st(ASEG, j, w.ld(ASEG, i));
-                w.st(ALEN, j, w.ld(ALEN, i));
-              }
+              if (i < n - 1) w.set_segment(j, w.segment(i));
             };
             if (up)
               for (int i = n - 1; i >= max(a0, W - 1); --i) move_any(i, i + 1);
-            {
+            if constexpr (!kTree) {
+              // two entries per pass, both read before either is written (the
+              // second entry's destination is the first one's source); the
+              // end vertex has no segment, what moves in its place is not read
+              const int d = up ? 1 : -1;
+              const int hi = min(n - 1, up ? W - 2 : W - 1);
+              const int cnt = hi - a0 + 1;
+              float4* sa = w.va(up ? hi : a0);
+              float2* sb = w.vb(up ? hi : a0);
+              float* sg = kGrad ? w.at(AGT, up ? hi : a0) : nullptr;
+              int t = 0;
+              for (; t + 1 < cnt; t += 2) {
+                const float4 v0 = sa[0], v1 = sa[-32 * d];
+                const float2 s0 = sb[0], s1 = sb[-32 * d];
+                const float g0 = kGrad ? sg[0] : 0.f, g1 = kGrad ? sg[-32 * d] : 0.f;
+                sa[32 * d] = v0;
+                sa[0] = v1;
+                sb[32 * d] = s0;
+                sb[0] = s1;
+                if constexpr (kGrad) {
+                  sg[32 * d] = g0;
+                  sg[0] = g1;
+                  sg -= 64 * d;
+                }
+                sa -= 64 * d;
+                sb -= 64 * d;
+              }
+              if (t < cnt) {
+                sa[32 * d] = sa[0];
+                sb[32 * d] = sb[0];
+                if constexpr (kGrad) sg[32 * d] = sg[0];
+              }
+            } else {
               const int d = up ? 1 : -1;
               const int hi = min(n - 1, up ? W - 2 : W - 1);
               const int cnt = hi - a0 + 1;
               const int WS = W * kRow;
-              float* src = w.row(up ? hi : a0);
+              float* src = w.at(AX, up ? hi : a0);
               int t = 0;
-              // two entries per pass, both read before either is written (the
-              // second entry's destination is the first one's source)
+              // two entries per pass, both read before either is written
               for (; t + 1 < cnt; t += 2, src -= 2 * d * kRow) {
                 float* src2 = src - d * kRow;
                 const float x0 = src[AX * WS], y0 = src[AY * WS], z0 = src[AZ * WS], v0 = src[AVT * WS];
@@ -709,10 +842,7 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
             if (v < nc) {
               w.st(AVT, wlo + v, nvt[v]);
               if constexpr (kGrad) w.st(AGT, wlo + v, ngt[v]);
-              if (v < nc - 1 && v < 2) {
-                w.st(ASEG, wlo + v, nseg[v]);
-                w.st(ALEN, wlo + v, nlen[v]);
-              }
+              if (v < nc - 1 && v < 2) w.set_segment(wlo + v, make_float2(nseg[v], nlen[v]));
             }
           }
           if (move != MV_DEATH) w.set_pos(inew, fnew);
@@ -780,9 +910,10 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
   acc[ACC_ACC + 2] += static_cast<double>(A.acc_b);
   acc[ACC_ACC + 3] += static_cast<double>(A.acc_d);
   for (int i = 0; i < min(n, W); ++i) {
-    w.gm[AX * cap + i] = w.sm[(AX * W + i) * kRow];
-    w.gm[AY * cap + i] = w.sm[(AY * W + i) * kRow];
-    w.gm[AZ * cap + i] = w.sm[(AZ * W + i) * kRow];
+    const float3 f = w.pos(i);
+    w.gm[AX * cap + i] = f.x;
+    w.gm[AY * cap + i] = f.y;
+    w.gm[AZ * cap + i] = f.z;
   }
   P.n[c] = n;
   P.step[c] = t_end;
