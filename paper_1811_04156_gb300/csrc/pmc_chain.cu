@@ -473,6 +473,7 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
     float* gz = gy + cap;
     w.gm = gx;
     w.cap = cap;
+    const WarpPath<kGen, kGrad, false> w_in{w.sm, w.gm, w.S, w.cap, w.b};  // the same path, all of it in the window
     float lam = 0.f;
     if constexpr (kLam) {
       lam = P.lam[c];
@@ -528,8 +529,8 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
         A.prop_d += __popc(__ballot_sync(kFull, live && type == 3u));
       }
       const int cnt = static_cast<int>(min(32ull, P.n_steps - s0));
-#pragma unroll 1
-      for (int i = 0; i < cnt; ++i) {
+      // one step on the path view `w`
+      auto step = [&](const auto& w, const int i) {
         const uint4 lo = rng[2 * i];
         const uint4 hi = rng[2 * i + 1];
         const uint32_t mtype = lo.x >> 24;
@@ -567,7 +568,7 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
               if (A.nflush >= kFlushAccepts) flush64(A, lane);
             }
             __syncwarp();
-            continue;
+            return;
           }
         }
         if constexpr (kTree) {
@@ -601,7 +602,7 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
               if (A.nflush >= kFlushAccepts) flush64(A, lane);
             }
             __syncwarp();
-            continue;
+            return;
           }
         }
         if constexpr (kLam) {
@@ -633,7 +634,7 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
               if (A.nflush >= kFlushAccepts) flush64(A, lane);
             }
             __syncwarp();
-            continue;
+            return;
           }
         }
         if (!kTree && mtype == 0u) {
@@ -821,6 +822,17 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
           L += dlen;
           G += dg;
           if (A.nflush >= kFlushAccepts) flush64(A, lane);
+        }
+      };
+#pragma unroll 1
+      for (int i = 0; i < cnt; ++i) {
+        if constexpr (kSpill) {
+          // a path that stays within the window even after a birth needs no
+          // test at its accesses
+          if (n < cap_s) step(w_in, i);
+          else step(w, i);
+        } else {
+          step(w, i);
         }
       }
       done += cnt;
