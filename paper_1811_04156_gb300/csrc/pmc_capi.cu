@@ -94,7 +94,7 @@ struct pmc_ctx_s {
   int n_sm = 0;
   size_t smem_per_sm = 0, smem_per_block = 0;
   // autotuned warps per block, keyed by (kernel instantiation, shared vertex cap, chain-count bucket)
-  std::map<std::tuple<int, int, int>, std::tuple<int, int, int>> tuned;  // -> (warps per block, shared window, kind)
+  std::map<std::tuple<int, int, int>, std::tuple<int, int, int, int>> tuned;  // -> (warps per block, window, kind, share)
 };
 
 struct pmc_medium_s {
@@ -170,7 +170,9 @@ struct pmc_geom_s {
 
 struct ChainClass {
   int kind = 0;       // kernel kind of launch_chain (4: one lane per chain)
+  int share = 0;      // kinds 0 and 1: how a warp's lanes share its chains (kShareGroup)
   bool short_paths = false;  // every pair expects <= kLaneMaxN vertices (lane layout candidate)
+  int expect_n = 0;   // vertices of the class's longest straight source-sensor line: 2 + its scattering depth
   int smem_cap = 0;   // shared window (vertices per chain)
   int max_cap = 0;    // largest vertex cap of the class's chains
   bool spill = false; // smem_cap < max_cap: entries beyond the window live in global memory
@@ -618,8 +620,11 @@ int pmc_destroy_chains(pmc_chains_t ch) {
 // states cannot see this, since those paths have not grown yet.
 constexpr double kLaneMaxN = 24.0;
 
-// Work items of a launch: one per chain, or one per 32 chains (lane layout).
-static int work_items(int kind, int chains) { return lane_kind(kind) ? (chains + 31) / 32 : chains; }
+// Work items of a launch: one per chain, per 32 chains (lane layout) or per warp of lane groups.
+static int work_items(int kind, int share, int chains) {
+  const int per_item = lane_kind(kind) ? 32 : (share == kShareGroup ? 32 / kGroupLanes : 1);
+  return (chains + per_item - 1) / per_item;
+}
 
 static ChainParams class_params(pmc_chains_t ch, size_t k, unsigned long long n_steps) {
   const ChainClass& cl = ch->classes[k];
@@ -658,19 +663,30 @@ static ChainParams class_params(pmc_chains_t ch, size_t k, unsigned long long n_
 // 128, 36.3 with 192, 30.8 with 256, 29.8 with 320.
 static int warp_window(pmc_chains_t ch, int full) {
   int most = 0;
-  if (chain_occupancy(ch->general, ch->grad, full > 32, 4, 32, &most) != cudaSuccess) return full;
+  if (chain_occupancy(ch->general, 0, ch->grad, full > 32, 4, 32, &most) != cudaSuccess) return full;
   for (int w = full; w > 32; w -= 32) {
     int bps = 0;
-    if (chain_smem_bytes(w, 4, ch->general, ch->grad) <= ch->ctx->smem_per_block &&
-        chain_occupancy(ch->general, ch->grad, w < full, 4, w, &bps) == cudaSuccess && bps >= most)
+    if (chain_smem_bytes(w, 4, ch->general, 0, ch->grad) <= ch->ctx->smem_per_block &&
+        chain_occupancy(ch->general, 0, ch->grad, w < full, 4, w, &bps) == cudaSuccess && bps >= most)
       return w;
   }
   return std::min(full, 32);
 }
 
+// When several chains share a warp.
+// Groups: the general physics with more chains than warps fit (20 per SM; 2,400
+// chains 0.98 ms with one warp per chain and 1.28 in groups, 3,600 1.74 and 1.39),
+// whose paths are expected to stay within the groups' window (the straight
+// line's vertex count); 30,720 chains of 44 vertices in 100 layers, 500 steps:
+// 10.3 ms with one warp per chain (window 256), 6.9 ms in groups (window 128;
+// 8.4 with 96, 9.3 with 192).  The lean kernel's longer paths spill there
+// (40 against 30 ms).
+constexpr int kGroupChains = 20, kGroupWindow = 128;
+
 // Autotuner: for every cap class, time the chain kernel over candidate launch
 // shapes — 1, 2 or 4 warps per block; with one warp per chain the shared
-// window of warp_window (entries beyond it in global memory); with one lane per chain (lean runs with short paths) a
+// window of warp_window (entries beyond it in global memory), or groups of 8
+// lanes per chain (rules above); with one lane per chain (lean runs with short paths) a
 // per-lane window of 8 to 32 vertices — on a scratch copy of the freshly initialised
 // state (256 steps, best of two probes), and keep the fastest; choices are
 // cached per device, kernel, layout request and class.
@@ -682,14 +698,16 @@ static int autotune_classes(pmc_chains_t ch, cudaStream_t s) {
   double* sacc = nullptr;
   int* sstat = nullptr;
   float* slam = nullptr;  // wavelength sampling: the probes' copy of the wavelengths
-  // cache key: the warp kernel instance, the layout request and which lane
-  // kernel (if any) the run may use; per class also whether its paths are short
-  const int kind = (((ch->general * 2 + ch->grad) * 3 + ch->layout) * 16 + ch->lane_kind) * 2;
+  // cache key: the warp kernel instance, the layout request, which lane kernel
+  // (if any) the run may use and whether its vertex moves are Gaussian; per
+  // class also whether its paths are short and whether they fit a group's window
+  const int kind = ((((ch->general * 2 + ch->grad) * 3 + ch->layout) * 16 + ch->lane_kind) * 2 +
+                    (ch->run.within == PMC_WITHIN_PERTURB)) * 4;
+  auto kind_of = [&](const ChainClass& cl) { return kind + cl.short_paths + 2 * (cl.expect_n <= kGroupWindow); };
   auto bucket_of = [](int chains) { return 31 - __builtin_clz(static_cast<unsigned>(std::max(1, chains))); };
   bool need = false;
   for (auto& cl : ch->classes)
-    if (!ch->ctx->tuned.count(std::make_tuple(kind + cl.short_paths, cl.max_cap, bucket_of(cl.hi - cl.lo))))
-      need = true;
+    if (!ch->ctx->tuned.count(std::make_tuple(kind_of(cl), cl.max_cap, bucket_of(cl.hi - cl.lo)))) need = true;
   if (need) {
     CK(dalloc(&sx, static_cast<size_t>(ch->xyz_floats)));
     CK(dalloc(&sn, T));
@@ -706,9 +724,9 @@ static int autotune_classes(pmc_chains_t ch, cudaStream_t s) {
     ChainClass& cl = ch->classes[k];
     const int chains = cl.hi - cl.lo;
     const int full = (cl.max_cap + 31) / 32 * 32;
-    const auto key = std::make_tuple(kind + cl.short_paths, cl.max_cap, bucket_of(chains));
+    const auto key = std::make_tuple(kind_of(cl), cl.max_cap, bucket_of(chains));
     auto it = ch->ctx->tuned.find(key);
-    std::tuple<int, int, int> best(cl.warps_per_block, cl.smem_cap, cl.kind);
+    std::tuple<int, int, int, int> best(cl.warps_per_block, cl.smem_cap, cl.kind, cl.share);
     if (it != ch->ctx->tuned.end()) {
       best = it->second;
     } else {
@@ -719,27 +737,30 @@ static int autotune_classes(pmc_chains_t ch, cudaStream_t s) {
         bool resident;  // the grid holds every work item at once
       };
       std::vector<LaneProbe> lane_probes;
-      // candidates (kind, shared window): the warp layout (tree and HMC moves
-      // keep the whole cap in shared memory); the lane layout (lean runs with short paths) with per-lane
+      // candidates (kind, shared window, sharing): the warp layout (tree and
+      // HMC moves keep the whole cap in shared memory); the lane layout (lean runs with short paths) with per-lane
       // windows of 8 to 32 vertices
-      std::vector<std::pair<int, int>> cands;
+      std::vector<std::tuple<int, int, int>> cands;
       if (ch->layout != PMC_LAYOUT_LANE) {
-        cands.emplace_back(ch->general, ch->general < 2 ? warp_window(ch, full) : full);
+        cands.emplace_back(ch->general, ch->general < 2 ? warp_window(ch, full) : full, 0);
+        if (ch->general == 1 && ch->run.within == PMC_WITHIN_PERTURB && chains >= kGroupChains * ch->ctx->n_sm &&
+            cl.expect_n <= kGroupWindow)
+          cands.assign(1, std::make_tuple(ch->general, std::min(full, kGroupWindow), kShareGroup));
       }
       if (ch->layout == PMC_LAYOUT_LANE ||
           (ch->layout == PMC_LAYOUT_AUTO && ch->lane_kind != 0 && cl.short_paths))
         for (int w : {8, 12, 16, 20, 24, 32}) {
-          cands.emplace_back(ch->lane_kind, std::min(w, cl.max_cap));
+          cands.emplace_back(ch->lane_kind, std::min(w, cl.max_cap), 0);
           if (w >= cl.max_cap) break;
         }
       for (const auto& cand : cands) {
-        const int ckind = cand.first, win = cand.second;
+        const int ckind = std::get<0>(cand), win = std::get<1>(cand), share = std::get<2>(cand);
         for (int wpb : {1, 2, 4}) {
           const bool spill = !lane_kind(ckind) && win < full;
-          if (chain_smem_bytes(win, wpb, ckind, ch->grad) > ch->ctx->smem_per_block) continue;
+          if (chain_smem_bytes(win, wpb, ckind, share, ch->grad) > ch->ctx->smem_per_block) continue;
           int bps = 0;
-          if (chain_occupancy(ckind, ch->grad, spill, wpb, win, &bps) != cudaSuccess || bps < 1) continue;
-          const int grid = std::max(1, std::min((work_items(ckind, chains) + wpb - 1) / wpb, bps * ch->ctx->n_sm));
+          if (chain_occupancy(ckind, share, ch->grad, spill, wpb, win, &bps) != cudaSuccess || bps < 1) continue;
+          const int grid = std::max(1, std::min((work_items(ckind, share, chains) + wpb - 1) / wpb, bps * ch->ctx->n_sm));
           ChainParams p = class_params(ch, k, 256);
           p.smem_cap = win;
           p.xyz = sx;
@@ -763,7 +784,7 @@ static int autotune_classes(pmc_chains_t ch, cudaStream_t s) {
               e = cudaMemcpyAsync(slam, ch->d_lam, sizeof(float) * T, cudaMemcpyDeviceToDevice, s);
             if (e == cudaSuccess) e = cudaMemsetAsync(ch->d_queue + k, 0, sizeof(unsigned int), s);
             if (e == cudaSuccess) e = cudaEventRecord(e0, s);
-            if (e == cudaSuccess) e = launch_chain(p, ckind, ch->grad, spill, grid, wpb, s);
+            if (e == cudaSuccess) e = launch_chain(p, ckind, share, ch->grad, spill, grid, wpb, s);
             if (e == cudaSuccess) e = cudaEventRecord(e1, s);
             if (e == cudaSuccess) e = cudaEventSynchronize(e1);
             float t = 0.f;
@@ -776,10 +797,10 @@ static int autotune_classes(pmc_chains_t ch, cudaStream_t s) {
           }
           if (ms < best_ms) {
             best_ms = ms;
-            best = std::make_tuple(wpb, win, ckind);
+            best = std::make_tuple(wpb, win, ckind, share);
           }
           if (lane_kind(ckind))
-            lane_probes.push_back({ms, wpb, win, ckind, (work_items(ckind, chains) + wpb - 1) / wpb <= grid});
+            lane_probes.push_back({ms, wpb, win, ckind, (work_items(ckind, share, chains) + wpb - 1) / wpb <= grid});
         }
         if (rc != PMC_OK) break;
       }
@@ -797,19 +818,20 @@ static int autotune_classes(pmc_chains_t ch, cudaStream_t s) {
           if (!keep || std::make_tuple(pr.resident, pr.win, -pr.ms) > std::make_tuple(keep->resident, keep->win, -keep->ms))
             keep = &pr;
         }
-        if (keep) best = std::make_tuple(keep->wpb, keep->win, keep->kind);
+        if (keep) best = std::make_tuple(keep->wpb, keep->win, keep->kind, 0);
       }
       if (rc == PMC_OK) ch->ctx->tuned[key] = best;
     }
     int bps = 0;
-    const int bw = std::get<0>(best), bwin = std::get<1>(best), bkind = std::get<2>(best);
+    const int bw = std::get<0>(best), bwin = std::get<1>(best), bkind = std::get<2>(best), bshare = std::get<3>(best);
     const bool spill = !lane_kind(bkind) && bwin < full;
-    if (rc == PMC_OK && chain_occupancy(bkind, ch->grad, spill, bw, bwin, &bps) == cudaSuccess && bps >= 1) {
+    if (rc == PMC_OK && chain_occupancy(bkind, bshare, ch->grad, spill, bw, bwin, &bps) == cudaSuccess && bps >= 1) {
       cl.kind = bkind;
+      cl.share = bshare;
       cl.warps_per_block = bw;
       cl.smem_cap = bwin;
       cl.spill = spill;
-      cl.grid = std::max(1, std::min((work_items(bkind, chains) + bw - 1) / bw, bps * ch->ctx->n_sm));
+      cl.grid = std::max(1, std::min((work_items(bkind, bshare, chains) + bw - 1) / bw, bps * ch->ctx->n_sm));
     }
   }
   cudaEventDestroy(e0);
@@ -978,7 +1000,8 @@ int pmc_init_chains(pmc_ctx_t ctx, pmc_medium_t med, pmc_geom_t geom, const pmc_
     const int k = class_key(ch->h_pairs[ch->h_pair_of[order[lo]]].cap);
     int hi = lo;
     int maxcap = 0;
-    double max_n = 0.0;
+    double max_n = 0.0, expect_n = 0.0;
+    int last_pair = -1;
     while (hi < T && class_key(ch->h_pairs[ch->h_pair_of[order[hi]]].cap) == k) {
       const DPair& d = ch->h_pairs[ch->h_pair_of[order[hi]]];
       maxcap = std::max(maxcap, d.cap);
@@ -986,6 +1009,9 @@ int pmc_init_chains(pmc_ctx_t ctx, pmc_medium_t med, pmc_geom_t geom, const pmc_
       const double dy = (static_cast<double>(d.c[1]) + d.c_lo[1]) - d.src[1];
       const double dz = (static_cast<double>(d.c[2]) + d.c_lo[2]) - d.src[2];
       max_n = std::max(max_n, 2.0 + std::sqrt(dx * dx + dy * dy + dz * dz) * med->d.b);
+      const int pair = ch->h_pair_of[order[hi]];
+      if (pair != last_pair) expect_n = std::max(expect_n, 2.0 + straight_tau_b(med, geom->host[pair]));
+      last_pair = pair;
       ++hi;
     }
     ChainClass cl;
@@ -993,6 +1019,7 @@ int pmc_init_chains(pmc_ctx_t ctx, pmc_medium_t med, pmc_geom_t geom, const pmc_
     cl.short_paths = med->d.kind == PMC_HOMOGENEOUS && max_n <= kLaneMaxN;
     cl.smem_cap = (maxcap + 31) / 32 * 32;
     cl.max_cap = maxcap;
+    cl.expect_n = static_cast<int>(std::min(expect_n, 1e6));
     cl.spill = false;
     if (r->layout == PMC_LAYOUT_LANE) {
       cl.kind = ch->lane_kind;
@@ -1015,20 +1042,20 @@ int pmc_init_chains(pmc_ctx_t ctx, pmc_medium_t med, pmc_geom_t geom, const pmc_
   for (auto& cl : ch->classes) {
     int wpb = r->warps_per_block > 0 ? r->warps_per_block : 4;
     wpb = std::min(wpb, 4);
-    while (wpb > 1 && chain_smem_bytes(cl.smem_cap, wpb, cl.kind, ch->grad) > ctx->smem_per_block) wpb /= 2;
-    if (chain_smem_bytes(cl.smem_cap, wpb, cl.kind, ch->grad) > ctx->smem_per_block) return fail(PMC_ERR_INVALID, "vertex cap too large for shared memory");
+    while (wpb > 1 && chain_smem_bytes(cl.smem_cap, wpb, cl.kind, cl.share, ch->grad) > ctx->smem_per_block) wpb /= 2;
+    if (chain_smem_bytes(cl.smem_cap, wpb, cl.kind, cl.share, ch->grad) > ctx->smem_per_block) return fail(PMC_ERR_INVALID, "vertex cap too large for shared memory");
     int bps = 0;
-    CK(chain_occupancy(cl.kind, ch->grad, cl.spill, wpb, cl.smem_cap, &bps));
+    CK(chain_occupancy(cl.kind, cl.share, ch->grad, cl.spill, wpb, cl.smem_cap, &bps));
     if (bps < 1) return fail(PMC_ERR_INVALID, "chain kernel does not fit on an SM");
     if (lane_kind(cl.kind) && r->warps_per_block <= 0) {
       // a lane-layout window set without warps per block: the shape that
       // keeps the most work items resident at once (the larger CTA on a
       // tie), since items beyond the resident warps run after the others
-      const int items = work_items(cl.kind, cl.hi - cl.lo);
+      const int items = work_items(cl.kind, cl.share, cl.hi - cl.lo);
       long best_res = static_cast<long>(std::min((items + wpb - 1) / wpb, bps * ctx->n_sm)) * wpb;
       for (int w2 = wpb / 2; w2 >= 1; w2 /= 2) {
         int b2 = 0;
-        CK(chain_occupancy(cl.kind, ch->grad, cl.spill, w2, cl.smem_cap, &b2));
+        CK(chain_occupancy(cl.kind, cl.share, ch->grad, cl.spill, w2, cl.smem_cap, &b2));
         if (b2 < 1) continue;
         const long res = static_cast<long>(std::min((items + w2 - 1) / w2, b2 * ctx->n_sm)) * w2;
         if (res > best_res) {
@@ -1038,7 +1065,7 @@ int pmc_init_chains(pmc_ctx_t ctx, pmc_medium_t med, pmc_geom_t geom, const pmc_
         }
       }
     }
-    const int want = (work_items(cl.kind, cl.hi - cl.lo) + wpb - 1) / wpb;
+    const int want = (work_items(cl.kind, cl.share, cl.hi - cl.lo) + wpb - 1) / wpb;
     cl.warps_per_block = wpb;
     cl.grid = std::max(1, std::min(want, bps * ctx->n_sm));
   }
@@ -1242,7 +1269,7 @@ static int enqueue_steps(pmc_chains_t ch, unsigned long long n_steps, cudaStream
   for (size_t k = 0; k < ch->classes.size(); ++k) {
     const ChainClass& cl = ch->classes[k];
     CK(cudaMemsetAsync(ch->d_queue + k, 0, sizeof(unsigned int), s));
-    CK(launch_chain(class_params(ch, k, n_steps), cl.kind, ch->grad, cl.spill, cl.grid, cl.warps_per_block, s));
+    CK(launch_chain(class_params(ch, k, n_steps), cl.kind, cl.share, ch->grad, cl.spill, cl.grid, cl.warps_per_block, s));
   }
   return PMC_OK;
 }

@@ -988,7 +988,8 @@ int kernel_key(int kind, bool grad, bool spill) {
 
 int chain_arrays(bool general, bool grad) { return 6 + (general ? 1 : 0) + (grad ? 1 : 0); }
 
-size_t chain_smem_bytes(int smem_cap, int warps_per_block, int kind, bool grad) {
+size_t chain_smem_bytes(int smem_cap, int warps_per_block, int kind, int share, bool grad) {
+  if (share == kShareGroup) return group_smem_bytes(grad, smem_cap, warps_per_block);
   if (lane_kind(kind)) return lane_smem_bytes(smem_cap, warps_per_block, grad, kind == 8);
   const size_t arrays = static_cast<size_t>(chain_arrays(kind > 0 && kind != 7, grad) + (kind == 2 || kind == 7 ? 3 : 0) +
                                             (kind == 3 ? 6 : 0));
@@ -997,12 +998,15 @@ size_t chain_smem_bytes(int smem_cap, int warps_per_block, int kind, bool grad) 
          sizeof(float);
 }
 
-cudaError_t chain_occupancy(int kind, bool grad, bool spill, int warps_per_block, int smem_cap,
+cudaError_t chain_occupancy(int kind, int share, bool grad, bool spill, int warps_per_block, int smem_cap,
                             int* blocks_per_sm) {
+  if (share == kShareGroup)
+    return kind == 1 ? group_kernel(grad, spill, nullptr, 0, warps_per_block, smem_cap, blocks_per_sm, nullptr)
+                     : cudaErrorInvalidValue;
   if (lane_kind(kind)) return lane_occupancy(kind, warps_per_block, smem_cap, grad, blocks_per_sm);
   if (kind >= 2 && spill) return cudaErrorInvalidValue;
   if (kind == 6 && grad) return cudaErrorInvalidValue;
-  const size_t sm = chain_smem_bytes(smem_cap, warps_per_block, kind, grad);
+  const size_t sm = chain_smem_bytes(smem_cap, warps_per_block, kind, share, grad);
   switch (kernel_key(kind, grad, spill)) {
     case 0: return occupancy_of<false, false, false, 0>(warps_per_block, sm, blocks_per_sm);
     case 1: return occupancy_of<false, false, true, 0>(warps_per_block, sm, blocks_per_sm);
@@ -1022,12 +1026,15 @@ cudaError_t chain_occupancy(int kind, bool grad, bool spill, int warps_per_block
   }
 }
 
-cudaError_t launch_chain(const ChainParams& p, int kind, bool grad, bool spill, int grid, int warps_per_block,
-                         cudaStream_t s) {
+cudaError_t launch_chain(const ChainParams& p, int kind, int share, bool grad, bool spill, int grid,
+                         int warps_per_block, cudaStream_t s) {
+  if (share == kShareGroup)
+    return kind == 1 ? group_kernel(grad, spill, &p, grid, warps_per_block, p.smem_cap, nullptr, s)
+                     : cudaErrorInvalidValue;
   if (lane_kind(kind)) return launch_lane_chain(p, kind, grid, warps_per_block, grad, s);
   if (kind >= 2 && spill) return cudaErrorInvalidValue;
   if (kind == 6 && grad) return cudaErrorInvalidValue;
-  const size_t sm = chain_smem_bytes(p.smem_cap, warps_per_block, kind, grad);
+  const size_t sm = chain_smem_bytes(p.smem_cap, warps_per_block, kind, share, grad);
   switch (kernel_key(kind, grad, spill)) {
     case 0: launch_one<false, false, false, 0>(p, grid, warps_per_block, sm, s); break;
     case 1: launch_one<false, false, true, 0>(p, grid, warps_per_block, sm, s); break;

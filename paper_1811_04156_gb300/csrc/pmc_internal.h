@@ -87,12 +87,22 @@ inline bool lane_kind(int kind) { return kind == 4 || kind == 5 || kind == 8; }
 // z and the per-vertex terms of its acceptance ratio), after the lane
 // layout's own in the chain's global block
 constexpr int kLaneTreeArrays = 4;
+// `share` (kinds 0 and 1): 0 one warp per chain; kShareGroup 8 lanes per chain
+// (kind 1, Gaussian moves; pmc_group.cuh).  The same decisions and the same
+// results.
+constexpr int kShareGroup = 1;
+constexpr int kGroupLanes = 8;
 int chain_arrays(bool general, bool grad);
-cudaError_t launch_chain(const ChainParams& p, int kind, bool grad, bool spill, int grid, int warps_per_block,
-                         cudaStream_t s);
-size_t chain_smem_bytes(int smem_cap, int warps_per_block, int kind, bool grad);
-cudaError_t chain_occupancy(int kind, bool grad, bool spill, int warps_per_block, int smem_cap,
+cudaError_t launch_chain(const ChainParams& p, int kind, int share, bool grad, bool spill, int grid,
+                         int warps_per_block, cudaStream_t s);
+size_t chain_smem_bytes(int smem_cap, int warps_per_block, int kind, int share, bool grad);
+cudaError_t chain_occupancy(int kind, int share, bool grad, bool spill, int warps_per_block, int smem_cap,
                             int* blocks_per_sm);
+
+// pmc_group.cu: launch, or occupancy when blocks_per_sm is given.
+size_t group_smem_bytes(bool grad, int smem_cap, int warps_per_block);
+cudaError_t group_kernel(bool grad, bool spill, const ChainParams* p, int grid, int warps_per_block, int smem_cap,
+                         int* blocks_per_sm, cudaStream_t s);
 
 // pmc_lane.cu (kinds 4, 5 and 8 above; `grad` adds the per-vertex d log
 // sigma / dg array, `tree` the proposed path's three arrays)

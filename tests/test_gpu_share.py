@@ -1,0 +1,57 @@
+"""Chain kernels in which several chains share a warp: the same chains, bit for
+bit, as the kernel with one warp per chain (which a request for warps per
+block selects), at ragged chain counts, paths on both sides of the shared
+window, step counts that end inside a batch, and split runs."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+from paper_1811_04156_gb300 import scenes as S
+
+pytestmark = pytest.mark.gpu
+
+
+def _run(scene, steps, **shape):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1811_04156_gb300 import api
+    ctx = api.Context(0)
+    medium = api.Medium(ctx, scene.medium)
+    geom = api.Geometry(ctx, scene.sources, scene.sensors, scene.pairs)
+    ch = api.Chains(ctx, medium, geom, scene.run, **shape)
+    for k in steps:
+        ch.run_steps(k)
+    return ch.launch_info()[0], ch.read_states(), ch.read_accumulators(), ch.status()
+
+
+def _same(a, b):
+    for x, y in zip(a[1], b[1]):
+        assert np.array_equal(x, y)
+    assert np.array_equal(a[2], b[2])
+    assert a[3] == b[3]  # (jittered straight starts that touch the sensor do not run)
+    assert (a[2][:, 0] > 0).sum() > 100
+
+
+@pytest.mark.parametrize("grad", [False, True])
+@pytest.mark.parametrize("init_k,cap", [(0, 40), (125, 200)])
+def test_lane_groups_match_one_warp_per_chain(grad, init_k, cap):
+    """General physics (layers, vMF emission, detection probability, phase
+    mixture), 8 lanes per chain; straight starts of 127 vertices grow and shrink
+    across the groups' window of 128."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    sc = S.general_small(n_chains=24 * n_sm + 3)
+    sc.pairs = [dataclasses.replace(sc.pairs[0], cap=cap)]
+    sc.run = dataclasses.replace(sc.run, gradients=grad, burn_in=50, p_birth=0.25, p_death=0.15, init_jitter=0.05,
+                                 init=S.INIT_STRAIGHT, init_k=init_k)
+    steps = (733, 35)
+    a = _run(sc, steps)
+    assert a[0]["general"] == 1 and a[0]["smem_cap"] == (128 if cap > 128 else 64)
+    _same(a, _run(sc, steps, warps_per_block=2))
+    if cap > 128:
+        assert a[1][1].max() > 128
+        _same(a, _run(sc, steps, warps_per_block=4, smem_window=64))
