@@ -170,7 +170,7 @@ struct pmc_geom_s {
 
 struct ChainClass {
   int kind = 0;       // kernel kind of launch_chain (4: one lane per chain)
-  int share = 0;      // kinds 0 and 1: how a warp's lanes share its chains (kShareGroup)
+  int share = 0;      // kinds 0 and 1: how a warp's lanes share its chains (kShareGroup, kShareTeam)
   bool short_paths = false;  // every pair expects <= kLaneMaxN vertices (lane layout candidate)
   int expect_n = 0;   // vertices of the class's longest straight source-sensor line: 2 + its scattering depth
   int smem_cap = 0;   // shared window (vertices per chain)
@@ -620,8 +620,10 @@ int pmc_destroy_chains(pmc_chains_t ch) {
 // states cannot see this, since those paths have not grown yet.
 constexpr double kLaneMaxN = 24.0;
 
-// Work items of a launch: one per chain, per 32 chains (lane layout) or per warp of lane groups.
+// Warps' work of a launch: one item per chain, per 32 chains (lane layout), per
+// warp of lane groups, or per warp of a team.
 static int work_items(int kind, int share, int chains) {
+  if (share == kShareTeam) return chains * 4;
   const int per_item = lane_kind(kind) ? 32 : (share == kShareGroup ? 32 / kGroupLanes : 1);
   return (chains + per_item - 1) / per_item;
 }
@@ -673,20 +675,24 @@ static int warp_window(pmc_chains_t ch, int full) {
   return std::min(full, 32);
 }
 
-// When several chains share a warp.
+// When several chains share a warp, or a team of warps works on one.
 // Groups: the general physics with more chains than warps fit (20 per SM; 2,400
 // chains 0.98 ms with one warp per chain and 1.28 in groups, 3,600 1.74 and 1.39),
 // whose paths are expected to stay within the groups' window (the straight
 // line's vertex count); 30,720 chains of 44 vertices in 100 layers, 500 steps:
 // 10.3 ms with one warp per chain (window 256), 6.9 ms in groups (window 128;
 // 8.4 with 96, 9.3 with 192).  The lean kernel's longer paths spill there
-// (40 against 30 ms).
-constexpr int kGroupChains = 20, kGroupWindow = 128;
+// (40 against 30 ms).  Teams: offered to the autotuner up to four chains per SM
+// (one warp per scheduler); 1,000 plain steps of 64 chains 0.94 ms with one warp
+// per chain, 0.75 with teams, of 608 chains 0.96 and 0.93, of 912 1.01 and 1.57
+// (100 layers: 1.39 and 1.16, 1.41 and 1.45, 1.49 and 2.55).
+constexpr int kGroupChains = 20, kGroupWindow = 128, kTeamChains = 4;
 
 // Autotuner: for every cap class, time the chain kernel over candidate launch
 // shapes — 1, 2 or 4 warps per block; with one warp per chain the shared
-// window of warp_window (entries beyond it in global memory), or groups of 8
-// lanes per chain (rules above); with one lane per chain (lean runs with short paths) a
+// window of warp_window (entries beyond it in global memory), four steps of a
+// chain per warp where the chains are few, or groups of 8 lanes per chain (rules
+// above); with one lane per chain (lean runs with short paths) a
 // per-lane window of 8 to 32 vertices — on a scratch copy of the freshly initialised
 // state (256 steps, best of two probes), and keep the fastest; choices are
 // cached per device, kernel, layout request and class.
@@ -743,6 +749,7 @@ static int autotune_classes(pmc_chains_t ch, cudaStream_t s) {
       std::vector<std::tuple<int, int, int>> cands;
       if (ch->layout != PMC_LAYOUT_LANE) {
         cands.emplace_back(ch->general, ch->general < 2 ? warp_window(ch, full) : full, 0);
+        if (ch->general < 2 && chains <= kTeamChains * ch->ctx->n_sm) cands.emplace_back(ch->general, full, kShareTeam);
         if (ch->general == 1 && ch->run.within == PMC_WITHIN_PERTURB && chains >= kGroupChains * ch->ctx->n_sm &&
             cl.expect_n <= kGroupWindow)
           cands.assign(1, std::make_tuple(ch->general, std::min(full, kGroupWindow), kShareGroup));
@@ -756,6 +763,7 @@ static int autotune_classes(pmc_chains_t ch, cudaStream_t s) {
       for (const auto& cand : cands) {
         const int ckind = std::get<0>(cand), win = std::get<1>(cand), share = std::get<2>(cand);
         for (int wpb : {1, 2, 4}) {
+          if (share == kShareTeam && wpb != 4) continue;
           const bool spill = !lane_kind(ckind) && win < full;
           if (chain_smem_bytes(win, wpb, ckind, share, ch->grad) > ch->ctx->smem_per_block) continue;
           int bps = 0;

@@ -50,6 +50,13 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
+// Teams of warps: what a warp tells the others about its step.
+constexpr int kTeamWarps = 4;
+struct TeamNote {
+  int what;        // bit 0: accepts, bit 1: an end move, from bit 2: the move kind
+  float dlen, dg;  // change of the path length and of the sum of d log sigma / dg
+};
+
 struct Sums {
   float L, G;
 };
@@ -411,13 +418,21 @@ __device__ __forceinline__ void flush64(Accum& a, int lane) {
 // CTAs of 128 threads per SM), which holds its out-of-line density call
 // without spills (+2 % on the two-sensor scene); the general Cartesian
 // kernel runs faster at 96 (-1 % at 128 on the layered workload).
+// kX = 4 is the Cartesian kernel with a team of four warps per chain, for runs
+// with too few chains to fill the GPU, where the latency of a step binds: warp
+// i evaluates step t + i of the chain, all from the same state.  Up to the
+// first accepted step the others were rejected, so their evaluations stand;
+// the first accepted one is committed and the next round starts after it.
+// With acceptance rate a, 1 + (1-a) + (1-a)^2 + (1-a)^3 steps finish per round.
+// (Four groups of 8 lanes of one warp instead of four warps gain little: they
+// run through each other's kinds of moves in turn.)
 template <bool kGen, bool kGrad, bool kSpill, int kX>
-__global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0) ? 5 : 6))
+__global__ void __launch_bounds__(128, (kGen && (kX == 1 || kX == 4)) ? 4 : ((kGen || kX != 0) ? 5 : 6))
     chain_kernel(const ChainParams P) {
   using WP = WarpPath<kGen, kGrad, kSpill>;
-  constexpr bool kTree = kX == 1, kHmc = kX == 2, kLam = kX == 3;
-  static_assert(kX == 0 || !kSpill, "tree, HMC and wavelength moves keep the whole cap in shared memory");
-  static_assert(kX == 0 || kX == 1 || kGen, "HMC and wavelength moves use the general kernel");
+  constexpr bool kTree = kX == 1, kHmc = kX == 2, kLam = kX == 3, kTeam = kX == 4;
+  static_assert(kX == 0 || !kSpill, "tree, HMC, wavelength and team kernels keep the whole cap in shared memory");
+  static_assert(kX == 0 || kX == 1 || kX == 4 || kGen, "HMC and wavelength moves use the general kernel");
   constexpr int kArraysAll = WP::kArrays + (kTree ? 3 : 0) + (kHmc ? 6 : 0);
   extern __shared__ float4 smem4[];
   float* smem = reinterpret_cast<float*>(smem4);
@@ -426,7 +441,7 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
   const int cap_s = P.smem_cap;
   const size_t per_warp = static_cast<size_t>(kArraysAll) * cap_s + 32 * kRngWords + kPairWords + (kLam ? kMedWords : 0);
   WP w;
-  w.sm = smem + static_cast<size_t>(wib) * per_warp;
+  w.sm = smem + (kTeam ? 0 : static_cast<size_t>(wib) * per_warp);
   w.S = cap_s;
   w.b = P.M.b;
   float* tnx = w.sm + static_cast<size_t>(WP::kArrays) * cap_s;  // tree / HMC moves: the proposed path
@@ -437,6 +452,14 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
   float* hmz = hmy + cap_s;
   uint4* rng = reinterpret_cast<uint4*>(w.sm + static_cast<size_t>(kArraysAll) * cap_s);  // [32][2] uint4
   DPair* spair = reinterpret_cast<DPair*>(rng + 64);
+  TeamNote* notes = nullptr;  // [2][kTeamWarps], by the round's parity
+  if constexpr (kTeam) {
+    // one path and one pair slot per block, random numbers per warp
+    spair = reinterpret_cast<DPair*>(rng + kTeamWarps * 64);
+    notes = reinterpret_cast<TeamNote*>(reinterpret_cast<float*>(spair) + kPairWords);
+    rng += wib * 64;
+  }
+  int parity = 0;
   // wavelength sampling: the medium at the chain's current wavelength, in the warp's shared slot
   DMedium* smed = reinterpret_cast<DMedium*>(reinterpret_cast<float*>(spair) + kPairWords);
   const DMedium& M = kLam ? *smed : P.M;
@@ -445,8 +468,16 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
 
   for (;;) {
     int item = 0;
-    if (lane == 0) item = static_cast<int>(atomicAdd(P.queue, 1u));
-    item = __shfl_sync(kFull, item, 0);
+    if constexpr (kTeam) {
+      __syncthreads();  // the block's previous chain is written back
+      if (threadIdx.x == 0) notes[0].what = static_cast<int>(atomicAdd(P.queue, 1u));
+      __syncthreads();
+      item = notes[0].what;
+      __syncthreads();
+    } else {
+      if (lane == 0) item = static_cast<int>(atomicAdd(P.queue, 1u));
+      item = __shfl_sync(kFull, item, 0);
+    }
     if (P.chain_lo + item >= P.chain_hi) break;
     const int c = P.order[P.chain_lo + item];
 
@@ -456,7 +487,8 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
       int* dst = reinterpret_cast<int*>(spair);
 #pragma unroll 1
       for (int q = lane; q < static_cast<int>(sizeof(DPair) / sizeof(int)); q += 32) dst[q] = src[q];
-      __syncwarp();
+      if constexpr (kTeam) __syncthreads();  // (each of a team's warps writes the same values)
+      else __syncwarp();
     }
     const DPair& S = *spair;
     const float zoff = S.zoff;
@@ -465,7 +497,7 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
     int n = P.n[c];
     const unsigned long long step0 = P.step[c];
     if (n < 2 || n > cap || (!kSpill && cap > cap_s)) {
-      if (lane == 0) { P.status[c] |= ST_BAD_N; atomicOr(P.any_status, ST_BAD_N); }
+      if (lane == 0 && (!kTeam || wib == 0)) { P.status[c] |= ST_BAD_N; atomicOr(P.any_status, ST_BAD_N); }
       continue;
     }
     float* gx = P.xyz + P.chain_base[c];
@@ -490,11 +522,12 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
     __syncwarp();
     const float lp0 = refresh_caches<kGen, kGen && kTree>(M, S, zoff, w, n, lane);
     if (!isfinite(lp0)) {
-      if (lane == 0) { P.status[c] |= ST_NONFINITE; atomicOr(P.any_status, ST_NONFINITE); }
+      if (lane == 0 && (!kTeam || wib == 0)) { P.status[c] |= ST_NONFINITE; atomicOr(P.any_status, ST_NONFINITE); }
       continue;
     }
     Sums sm = path_sums(w, n, lane);
     float L = sm.L, G = sm.G;
+    if constexpr (kTeam) __syncthreads();
 
     Accum A;
     A.pn2 = A.pn = 0;
@@ -511,7 +544,14 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
     unsigned long long done = 0;
     bool aborted = false;
     for (unsigned long long s0 = 0; s0 < P.n_steps; s0 += 32) {
-      if ((s0 & 1023ull) == 0 && P.abort_flag != nullptr && *P.abort_flag) { aborted = true; break; }
+      if ((s0 & 1023ull) == 0 && P.abort_flag != nullptr) {
+        // (a team stops together)
+        const bool stop = kTeam ? __syncthreads_or(*P.abort_flag != 0) != 0 : *P.abort_flag != 0;
+        if (stop) {
+          aborted = true;
+          break;
+        }
+      }
       // ---- lane-parallel random numbers of steps step0+s0 .. +31 ----
       {
         const unsigned long long tl = step0 + s0 + lane;
@@ -529,10 +569,13 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
         A.prop_d += __popc(__ballot_sync(kFull, live && type == 3u));
       }
       const int cnt = static_cast<int>(min(32ull, P.n_steps - s0));
-      // one step on the path view `w`
-      auto step = [&](const auto& w, const int i) {
-        const uint4 lo = rng[2 * i];
-        const uint4 hi = rng[2 * i + 1];
+      // step i of the batch on the path view `w`; a team's warps each take one
+      // (`live`: there is such a step), and the number of steps that their
+      // round finished is returned
+      auto step = [&](const auto& w, const int i, const bool live) -> int {
+        const int row = kTeam ? min(i, cnt - 1) : i;
+        const uint4 lo = rng[2 * row];
+        const uint4 hi = rng[2 * row + 1];
         const uint32_t mtype = lo.x >> 24;
         const uint32_t v23 = lo.x & 0x7fffffu;
         const float logu = __uint_as_float(lo.y);
@@ -568,7 +611,7 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
               if (A.nflush >= kFlushAccepts) flush64(A, lane);
             }
             __syncwarp();
-            return;
+            return 1;
           }
         }
         if constexpr (kTree) {
@@ -602,7 +645,7 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
               if (A.nflush >= kFlushAccepts) flush64(A, lane);
             }
             __syncwarp();
-            return;
+            return 1;
           }
         }
         if constexpr (kLam) {
@@ -634,7 +677,7 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
               if (A.nflush >= kFlushAccepts) flush64(A, lane);
             }
             __syncwarp();
-            return;
+            return 1;
           }
         }
         if (!kTree && mtype == 0u) {
@@ -643,7 +686,7 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
           inew = j;
           if (j == n - 1) {
             move = MV_END;
-            A.prop_end++;
+            if constexpr (!kTeam) A.prop_end++;
             const float3 nu = sensor_normal(S, w.pos(j));
             float3 e1, e2;
             onb(nu, e1, e2);
@@ -656,7 +699,7 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
             move = MV_INTERIOR;
             const float3 fj = w.pos(j);
             const float3 z = f3(__uint_as_float(lo.z), __uint_as_float(lo.w), __uint_as_float(hi.x));
-            if constexpr (kGen && kX == 0) {
+            if constexpr (kGen && (kX == 0 || kTeam)) {
               if (R.within == 1) {
                 gx_mala = grad_vertex_warp<32>(M, S, zoff, [&](int k) { return w.pos(k); }, n, j, lane);
                 const float h = 0.5f * R.mala_eps * R.mala_eps;
@@ -772,7 +815,7 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
             extra = -R.log_pd + __logf(static_cast<float>(n - 2)) + R.log_pb + __logf(__fdividef(tb_new, Tb_red)) +
                     log_insert_density<true>(M, R, zoff, w.pos(jj - 1), w.pos(jj + 1), w.pos(jj));
           }
-          if constexpr (kGen && kX == 0) {
+          if constexpr (kGen && (kX == 0 || kTeam)) {
             if (move == MV_INTERIOR && R.within == 1 && isfinite(dlp)) {
               const float3 gy = grad_vertex_warp<32>(M, S, zoff, newpos, n, jj, lane);
               const float h = 0.5f * R.mala_eps * R.mala_eps;
@@ -784,55 +827,94 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
           }
           accept = logu < dlp + extra;
         }
+        float dlen = 0.f, dg = 0.f;
         if (accept) {
-          A.acc_i += (move == MV_INTERIOR);
-          A.acc_e += (move == MV_END);
-          A.acc_b += (move == MV_BIRTH);
-          A.acc_d += (move == MV_DEATH);
-          close_state(A, t, R.burn_in, n, L, G);
-          float dlen = nlen - olen;
+          dlen = nlen - olen;
           dlen += __shfl_xor_sync(kFull, dlen, 1);
           dlen += __shfl_xor_sync(kFull, dlen, 2);
           dlen = __shfl_sync(kFull, dlen, 0);
-          float dg = 0.f;
           if constexpr (kGrad) {
             dg = ngt - ogt;
             dg += __shfl_xor_sync(kFull, dg, 1);
             dg += __shfl_xor_sync(kFull, dg, 2);
             dg = __shfl_sync(kFull, dg, 0);
           }
-          if (move == MV_BIRTH) {
-            shift_right(w, kk + 1, n, n - 1, lane);
-          } else if (move == MV_DEATH) {
-            shift_left(w, jj + 1, n, n - 1, lane);
+        }
+        unsigned long long t_acc = t;
+        int used = 1;
+        bool any = accept;  // the round ends with an accepted step
+        if constexpr (kTeam) {
+          TeamNote* note = notes + parity * kTeamWarps;
+          parity ^= 1;
+          accept = accept && live;
+          if (lane == 0) note[wib] = TeamNote{(accept ? 1 : 0) | (live && move == MV_END ? 2 : 0) | (move << 2), dlen, dg};
+          __syncthreads();
+          int chosen = kTeamWarps, ends = 0;
+#pragma unroll
+          for (int k = kTeamWarps - 1; k >= 0; --k)
+            if (note[k].what & 1) chosen = k;
+          any = chosen < kTeamWarps;
+          used = any ? chosen + 1 : kTeamWarps;
+#pragma unroll
+          for (int k = 0; k < kTeamWarps; ++k)
+            if (k < used) ends += (note[k].what >> 1) & 1;
+          A.prop_end += ends;
+          accept = any && chosen == wib;
+          if (any) {
+            t_acc = step0 + s0 + (i - wib) + chosen;
+            move = note[chosen].what >> 2;
+            dlen = note[chosen].dlen;
+            dg = note[chosen].dg;
+            n_new = n + (move == MV_BIRTH) - (move == MV_DEATH);
           }
-          if (lane < nc) {
-            const int v = wlo + lane;
-            w.set_vt(v, nvt);
-            w.set_gt(v, ngt);
-            if (lane < nc - 1) {
-              w.set_seg(v, nseg);
-              w.set_tb(v, ntb);
-              w.set_len(v, nlen);
+        }
+        if (any) {
+          A.acc_i += (move == MV_INTERIOR);
+          A.acc_e += (move == MV_END);
+          A.acc_b += (move == MV_BIRTH);
+          A.acc_d += (move == MV_DEATH);
+          close_state(A, t_acc, R.burn_in, n, L, G);
+          if (accept) {
+            if (move == MV_BIRTH) {
+              shift_right(w, kk + 1, n, n - 1, lane);
+            } else if (move == MV_DEATH) {
+              shift_left(w, jj + 1, n, n - 1, lane);
             }
+            if (lane < nc) {
+              const int v = wlo + lane;
+              w.set_vt(v, nvt);
+              w.set_gt(v, ngt);
+              if (lane < nc - 1) {
+                w.set_seg(v, nseg);
+                w.set_tb(v, ntb);
+                w.set_len(v, nlen);
+              }
+            }
+            if (lane == 0 && move != MV_DEATH) w.set_pos(inew, fnew);
           }
-          if (lane == 0 && move != MV_DEATH) w.set_pos(inew, fnew);
-          __syncwarp();
+          if constexpr (kTeam) __syncthreads();
+          else __syncwarp();
           n = n_new;
           L += dlen;
           G += dg;
           if (A.nflush >= kFlushAccepts) flush64(A, lane);
         }
+        return used;
       };
 #pragma unroll 1
-      for (int i = 0; i < cnt; ++i) {
+      for (int i = 0; i < cnt;) {
         if constexpr (kSpill) {
           // a path that stays within the window even after a birth needs no
           // test at its accesses
-          if (n < cap_s) step(w_in, i);
-          else step(w, i);
+          if (n < cap_s) step(w_in, i, true);
+          else step(w, i, true);
+          ++i;
+        } else if constexpr (kTeam) {
+          const int mine = i + wib;
+          i += step(w, mine, mine < cnt);
         } else {
-          step(w, i);
+          step(w, i, true);
+          ++i;
         }
       }
       done += cnt;
@@ -859,6 +941,7 @@ __global__ void __launch_bounds__(128, (kGen && kX == 1) ? 4 : ((kGen || kX != 0
     if (lane == ACC_ACC + 2) extra_w = static_cast<double>(A.acc_b);
     if (lane == ACC_ACC + 3) extra_w = static_cast<double>(A.acc_d);
     A.my += extra_w;
+    if (kTeam && wib != 0) continue;  // one of the team's warps writes back
     if (lane < ACC_WORDS) P.acc[static_cast<size_t>(c) * ACC_WORDS + lane] = A.my;
 #pragma unroll 1
     for (int i = lane; i < min(n, cap_s); i += 32) {
@@ -976,7 +1059,8 @@ void launch_one(const ChainParams& p, int grid, int warps_per_block, size_t sm, 
 
 // Instantiation key: lean / general (with or without gradient caches and
 // spill), general with tree moves and general with HMC moves (never spilled).
-int kernel_key(int kind, bool grad, bool spill) {
+int kernel_key(int kind, int share, bool grad, bool spill) {
+  if (share == kShareTeam) return 16 + (kind == 1 ? 2 : 0) + (grad ? 1 : 0);
   if (kind == 2) return 8 + (grad ? 1 : 0);
   if (kind == 3) return 10 + (grad ? 1 : 0);
   if (kind == 6) return 12;
@@ -990,6 +1074,9 @@ int chain_arrays(bool general, bool grad) { return 6 + (general ? 1 : 0) + (grad
 
 size_t chain_smem_bytes(int smem_cap, int warps_per_block, int kind, int share, bool grad) {
   if (share == kShareGroup) return group_smem_bytes(grad, smem_cap, warps_per_block);
+  if (share == kShareTeam)
+    return (static_cast<size_t>(chain_arrays(kind == 1, grad)) * smem_cap + kTeamWarps * 32u * kRngWords + kPairWords) *
+               sizeof(float) + 2 * kTeamWarps * sizeof(TeamNote);
   if (lane_kind(kind)) return lane_smem_bytes(smem_cap, warps_per_block, grad, kind == 8);
   const size_t arrays = static_cast<size_t>(chain_arrays(kind > 0 && kind != 7, grad) + (kind == 2 || kind == 7 ? 3 : 0) +
                                             (kind == 3 ? 6 : 0));
@@ -1003,11 +1090,12 @@ cudaError_t chain_occupancy(int kind, int share, bool grad, bool spill, int warp
   if (share == kShareGroup)
     return kind == 1 ? group_kernel(grad, spill, nullptr, 0, warps_per_block, smem_cap, blocks_per_sm, nullptr)
                      : cudaErrorInvalidValue;
+  if (share == kShareTeam && (kind > 1 || spill || warps_per_block != kTeamWarps)) return cudaErrorInvalidValue;
   if (lane_kind(kind)) return lane_occupancy(kind, warps_per_block, smem_cap, grad, blocks_per_sm);
   if (kind >= 2 && spill) return cudaErrorInvalidValue;
   if (kind == 6 && grad) return cudaErrorInvalidValue;
   const size_t sm = chain_smem_bytes(smem_cap, warps_per_block, kind, share, grad);
-  switch (kernel_key(kind, grad, spill)) {
+  switch (kernel_key(kind, share, grad, spill)) {
     case 0: return occupancy_of<false, false, false, 0>(warps_per_block, sm, blocks_per_sm);
     case 1: return occupancy_of<false, false, true, 0>(warps_per_block, sm, blocks_per_sm);
     case 2: return occupancy_of<false, true, false, 0>(warps_per_block, sm, blocks_per_sm);
@@ -1022,6 +1110,10 @@ cudaError_t chain_occupancy(int kind, int share, bool grad, bool spill, int warp
     case 12: return occupancy_of<true, false, false, 3>(warps_per_block, sm, blocks_per_sm);
     case 14: return occupancy_of<false, false, false, 1>(warps_per_block, sm, blocks_per_sm);
     case 15: return occupancy_of<false, true, false, 1>(warps_per_block, sm, blocks_per_sm);
+    case 16: return occupancy_of<false, false, false, 4>(warps_per_block, sm, blocks_per_sm);
+    case 17: return occupancy_of<false, true, false, 4>(warps_per_block, sm, blocks_per_sm);
+    case 18: return occupancy_of<true, false, false, 4>(warps_per_block, sm, blocks_per_sm);
+    case 19: return occupancy_of<true, true, false, 4>(warps_per_block, sm, blocks_per_sm);
     default: return occupancy_of<true, true, false, 2>(warps_per_block, sm, blocks_per_sm);
   }
 }
@@ -1031,11 +1123,12 @@ cudaError_t launch_chain(const ChainParams& p, int kind, int share, bool grad, b
   if (share == kShareGroup)
     return kind == 1 ? group_kernel(grad, spill, &p, grid, warps_per_block, p.smem_cap, nullptr, s)
                      : cudaErrorInvalidValue;
+  if (share == kShareTeam && (kind > 1 || spill || warps_per_block != kTeamWarps)) return cudaErrorInvalidValue;
   if (lane_kind(kind)) return launch_lane_chain(p, kind, grid, warps_per_block, grad, s);
   if (kind >= 2 && spill) return cudaErrorInvalidValue;
   if (kind == 6 && grad) return cudaErrorInvalidValue;
   const size_t sm = chain_smem_bytes(p.smem_cap, warps_per_block, kind, share, grad);
-  switch (kernel_key(kind, grad, spill)) {
+  switch (kernel_key(kind, share, grad, spill)) {
     case 0: launch_one<false, false, false, 0>(p, grid, warps_per_block, sm, s); break;
     case 1: launch_one<false, false, true, 0>(p, grid, warps_per_block, sm, s); break;
     case 2: launch_one<false, true, false, 0>(p, grid, warps_per_block, sm, s); break;
@@ -1050,6 +1143,10 @@ cudaError_t launch_chain(const ChainParams& p, int kind, int share, bool grad, b
     case 12: launch_one<true, false, false, 3>(p, grid, warps_per_block, sm, s); break;
     case 14: launch_one<false, false, false, 1>(p, grid, warps_per_block, sm, s); break;
     case 15: launch_one<false, true, false, 1>(p, grid, warps_per_block, sm, s); break;
+    case 16: launch_one<false, false, false, 4>(p, grid, warps_per_block, sm, s); break;
+    case 17: launch_one<false, true, false, 4>(p, grid, warps_per_block, sm, s); break;
+    case 18: launch_one<true, false, false, 4>(p, grid, warps_per_block, sm, s); break;
+    case 19: launch_one<true, true, false, 4>(p, grid, warps_per_block, sm, s); break;
     default: launch_one<true, true, false, 2>(p, grid, warps_per_block, sm, s); break;
   }
   return cudaGetLastError();

@@ -88,9 +88,10 @@ inline bool lane_kind(int kind) { return kind == 4 || kind == 5 || kind == 8; }
 // layout's own in the chain's global block
 constexpr int kLaneTreeArrays = 4;
 // `share` (kinds 0 and 1): 0 one warp per chain; kShareGroup 8 lanes per chain
-// (kind 1, Gaussian moves; pmc_group.cuh).  The same decisions and the same
-// results.
-constexpr int kShareGroup = 1;
+// (kind 1, Gaussian moves; pmc_group.cuh); kShareTeam a block of four warps per
+// chain, each on one of its next steps (no spill).  The same decisions and the
+// same results.
+constexpr int kShareGroup = 1, kShareTeam = 2;
 constexpr int kGroupLanes = 8;
 int chain_arrays(bool general, bool grad);
 cudaError_t launch_chain(const ChainParams& p, int kind, int share, bool grad, bool spill, int grid,
