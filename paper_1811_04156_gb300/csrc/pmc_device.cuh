@@ -362,7 +362,7 @@ __device__ __forceinline__ float3 drdot(float3 rhat, float ell, float3 w) {
 template <class PosF>
 __device__ float3 grad_vertex(const DMedium& M, const DPair& S, float zoff, PosF pos, int n, int v) {
   float3 rh[4];
-  float el[4];
+  float el[4], il[4];
   bool ex[4];
   float3 pv[5];
 #pragma unroll
@@ -376,19 +376,20 @@ __device__ float3 grad_vertex(const DMedium& M, const DPair& S, float zoff, PosF
     ex[i] = (k >= 0 && k <= n - 2);
     const float3 r = pv[i + 1] - pv[i];
     el[i] = ex[i] ? sqrtf(dot(r, r)) : 1.0f;
-    rh[i] = (1.0f / el[i]) * r;
+    il[i] = 1.0f / el[i];
+    rh[i] = il[i] * r;
   }
   float3 g = f3(0.f, 0.f, 0.f);
   // segment v-1 ends at v, segment v starts at v
   if (ex[1]) {
     float3 dP, dQ;
     dtau_dends(M, zoff, pv[1], pv[2], el[1], rh[1], dP, dQ);
-    g = g - dQ - (2.0f / el[1]) * rh[1];
+    g = g - dQ - (2.0f * il[1]) * rh[1];  // (2 il rounds as 2 / el does)
   }
   if (ex[2]) {
     float3 dP, dQ;
     dtau_dends(M, zoff, pv[2], pv[3], el[2], rh[2], dP, dQ);
-    g = g - dP + (2.0f / el[2]) * rh[2];
+    g = g - dP + (2.0f * il[2]) * rh[2];
   }
   // emission
   if (S.emission != 0) {

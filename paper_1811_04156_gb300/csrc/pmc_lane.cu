@@ -234,6 +234,7 @@ __device__ __forceinline__ void pooled_for(TreeSlot* slots, int count, F&& fn) {
   scan[lane] = incl;
   __syncwarp();
   int src = 0;
+#pragma unroll 1
   for (int f = lane; f < total; f += 32) {
     while (scan[src] <= f) ++src;
     fn(src, f - (src > 0 ? scan[src - 1] : 0));
@@ -274,6 +275,7 @@ __device__ float pooled_tree_gain(const ChainParams& P, TreeSlot* slots, float* 
   // and its parent's triangle), and +log of each volume element at x'
   const int levels = mine ? tree_levels(n_mine) : 0;
   const int depth = __reduce_max_sync(kAll, static_cast<unsigned>(levels));
+#pragma unroll 1
   for (int d = 0; d < depth; ++d) {
     pooled_for(slots, d < levels ? (1 << d) : 0, [&](int src, int j) {
       const TreeSlot& T = slots[src];
@@ -303,6 +305,7 @@ __device__ float pooled_tree_gain(const ChainParams& P, TreeSlot* slots, float* 
   float gain = 0.f;
   if (mine) {
     const Proposal q = proposal_of<kGrad>(slots[lane], pool);
+#pragma unroll 1
     for (int i = 0; i < n_mine; ++i) gain += q.ld(PG, i);
   }
   return gain;
@@ -340,6 +343,7 @@ __device__ void pooled_tree_commit(const ChainParams& P, TreeSlot* slots, float*
 template <bool kGrad, int kRow>
 __device__ __forceinline__ void lane_refresh_sums(const LanePath<kRow>& w, int n, float& L, float& G) {
   float Ls = 0.f;
+#pragma unroll (kRow == 33 ? 1 : 4)
   for (int q = 0; q < n - 1; ++q) Ls += w.ld(ALEN, q);
   L = Ls;
   if constexpr (kGrad) {
@@ -403,6 +407,7 @@ template <bool kGrad, bool kMala, bool kTree>
 __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own, float* col, int W, uint32_t key0,
                                           uint32_t key1, TreeSlot* slots, float* pool) {
   constexpr int kRow = row_of(kTree);
+  constexpr int kRoll = kTree ? 1 : 4;  // tree moves: loops rolled for the instruction cache
   const DMedium& M = P.M;
   const DRun& R = P.R;
   const int lane = threadIdx.x & 31;
@@ -571,6 +576,7 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
             cum += M.b * *w.at(ALEN, q);
             below += (cum <= target) ? 1 : 0;
           }
+#pragma unroll kRoll
           for (int q = W; q < n - 1; ++q) {
             cum += M.b * w.gm[ALEN * cap + q];
             below += (cum <= target) ? 1 : 0;
@@ -752,6 +758,7 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
               if (i < n - 1) w.set_segment(j, w.segment(i));
             };
             if (up)
+#pragma unroll kRoll
               for (int i = n - 1; i >= max(a0, W - 1); --i) move_any(i, i + 1);
             if constexpr (!kTree) {
               // two entries per pass, both read before either is written (the
@@ -793,6 +800,7 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
               float* src = w.at(AX, up ? hi : a0);
               int t = 0;
               // two entries per pass, both read before either is written
+#pragma unroll kRoll
               for (; t + 1 < cnt; t += 2, src -= 2 * d * kRow) {
                 float* src2 = src - d * kRow;
                 const float x0 = src[AX * WS], y0 = src[AY * WS], z0 = src[AZ * WS], v0 = src[AVT * WS];
@@ -835,6 +843,7 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
               }
             }
             if (!up)
+#pragma unroll kRoll
               for (int i = max(a0, W); i <= n - 1; ++i) move_any(i, i - 1);
           }
 #pragma unroll
@@ -874,6 +883,7 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
         bool taken = false;
         if (mine) {
           float lpo = 0.f;
+#pragma unroll 1
           for (int q = 0; q < n; ++q) lpo += w.ld(AVT, q) + ((q <= n - 2) ? w.ld(ASEG, q) : 0.f);
           taken = logu_mine < gain - lpo;
           if (taken) {
