@@ -46,7 +46,7 @@ struct SharedDivisor {
   }
 };
 
-// What the flights of lean photons share.
+// What the flights of a thread's photons share (b: lean photons only).
 struct FlightConsts {
   SharedDivisor by_b, by_2g;
   __device__ explicit FlightConsts(const DMedium& M) : by_b(M.b), by_2g(2.0f * M.g) {}
@@ -106,8 +106,7 @@ __device__ inline float draw_cos_theta(const DMedium& M, const FlightConsts& C, 
   const float g = M.g;
   if (!kLean && fabsf(g) < 1e-6f) return 2.0f * u - 1.0f;
   const float q = (1.0f - g * g) / (1.0f - g + 2.0f * g * u);
-  const float num = 1.0f + g * g - q * q;
-  return fminf(fmaxf(kLean ? C.by_2g.quotient(num) : num / (2.0f * g), -1.0f), 1.0f);
+  return fminf(fmaxf(C.by_2g.quotient(1.0f + g * g - q * q), -1.0f), 1.0f);
 }
 
 // Unit vector at polar cosine ct and azimuth (sin, cos) = (sp, cp) about axis.
