@@ -1273,11 +1273,18 @@ int pmc_set_states(pmc_chains_t ch, const float* xyz, const int* n, int stride, 
   return PMC_OK;
 }
 
+// One launch per cap class; the lane kernels count a launch's steps in 32 bits.
+constexpr unsigned long long kLaneLaunchSteps = 1ull << 30;
 static int enqueue_steps(pmc_chains_t ch, unsigned long long n_steps, cudaStream_t s) {
   for (size_t k = 0; k < ch->classes.size(); ++k) {
     const ChainClass& cl = ch->classes[k];
-    CK(cudaMemsetAsync(ch->d_queue + k, 0, sizeof(unsigned int), s));
-    CK(launch_chain(class_params(ch, k, n_steps), cl.kind, cl.share, ch->grad, cl.spill, cl.grid, cl.warps_per_block, s));
+    const unsigned long long most = lane_kind(cl.kind) ? kLaneLaunchSteps : n_steps;
+    for (unsigned long long left = n_steps; left > 0;) {
+      const unsigned long long now = std::min(left, most);
+      CK(cudaMemsetAsync(ch->d_queue + k, 0, sizeof(unsigned int), s));
+      CK(launch_chain(class_params(ch, k, now), cl.kind, cl.share, ch->grad, cl.spill, cl.grid, cl.warps_per_block, s));
+      left -= now;
+    }
   }
   return PMC_OK;
 }

@@ -129,24 +129,25 @@ struct LanePath {
 
 // Per-chain recording state: the current state's observables enter the sums
 // once, weighted by the steps it stayed current (at or after burn-in).
+// Steps count from the start of the launch, at most 2^30 of them.
 struct LaneAcc {
-  unsigned long long pn2, pn, t_a;
+  unsigned long long pn;
+  unsigned int pn2, t_a;
   float pL, pL2, pG;
   unsigned int nflush;
-  unsigned int prop_w, prop_end, prop_b, prop_d;
+  unsigned int prop_w, prop_end, prop_b;  // deaths: the other steps
   unsigned int acc_i, acc_e, acc_b, acc_d;
 };
 
 template <bool kGrad>
-__device__ __forceinline__ void lane_close(LaneAcc& a, unsigned long long t_b, unsigned long long burn_in, int n,
-                                           float L, float G) {
-  const unsigned long long from = a.t_a > burn_in ? a.t_a : burn_in;
+__device__ __forceinline__ void lane_close(LaneAcc& a, unsigned int t_b, unsigned int burn_in, int n, float L, float G) {
+  const unsigned int from = max(a.t_a, burn_in);
   a.t_a = t_b;
   if (t_b <= from) return;
-  const unsigned long long d = t_b - from;
+  const unsigned int d = t_b - from;
   const float dw = static_cast<float>(d);
-  a.pn2 += (n == 2) ? d : 0ull;
-  a.pn += static_cast<unsigned long long>(n) * d;
+  a.pn2 += (n == 2) ? d : 0u;
+  a.pn += static_cast<unsigned long long>(static_cast<unsigned int>(n)) * d;
   a.pL = fmaf(L, dw, a.pL);
   a.pL2 = fmaf(L * L, dw, a.pL2);
   if constexpr (kGrad) a.pG = fmaf(G, dw, a.pG);
@@ -160,7 +161,8 @@ __device__ __forceinline__ void lane_flush(LaneAcc& a, double* acc) {
   acc[ACC_SUML] += static_cast<double>(a.pL);
   acc[ACC_SUML2] += static_cast<double>(a.pL2);
   if constexpr (kGrad) acc[ACC_SUMG] += static_cast<double>(a.pG);
-  a.pn2 = a.pn = 0ull;
+  a.pn = 0ull;
+  a.pn2 = 0u;
   a.pL = a.pL2 = a.pG = 0.f;
   a.nflush = 0;
 }
@@ -466,11 +468,13 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
     own = false;
   }
   LaneAcc A;
-  A.pn2 = A.pn = 0ull;
-  A.t_a = step0;
+  A.pn = 0ull;
+  A.pn2 = A.t_a = 0u;
+  const unsigned int burn_in =  // burn-in steps of this launch
+      R.burn_in > step0 ? static_cast<unsigned int>(min(R.burn_in - step0, 0xffffffffull)) : 0u;
   A.pL = A.pL2 = A.pG = 0.f;
   A.nflush = 0;
-  A.prop_w = A.prop_end = A.prop_b = A.prop_d = 0;
+  A.prop_w = A.prop_end = A.prop_b = 0;
   A.acc_i = A.acc_e = A.acc_b = A.acc_d = 0;
   double* acc = P.acc + static_cast<size_t>(c) * ACC_WORDS;
   const float3 cS = f3(S.c[0], S.c[1], S.c[2]);
@@ -478,10 +482,11 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
   const uint32_t cid = static_cast<uint32_t>(c) + P.chain_id0;  // global chain index
   const float3 vref = kTree ? tree_vref(S) : f3(1.f, 0.f, 0.f);  // tree moves: the root frame's reference
   float* const cols = col - lane;                                 // the warp's columns
-  unsigned long long done = 0;
+  unsigned int done = 0;
   bool aborted = false;
-  for (unsigned long long s = 0; s < P.n_steps; ++s) {
-    if ((s & 1023ull) == 0 && P.abort_flag != nullptr) {
+  const unsigned int n_steps = static_cast<unsigned int>(P.n_steps);
+  for (unsigned int s = 0; s < n_steps; ++s) {
+    if ((s & 1023u) == 0 && P.abort_flag != nullptr) {
       // with tree moves the whole warp stops together (its pooled passes need every lane)
       bool stop;
       if constexpr (kTree) stop = __any_sync(kAll, *P.abort_flag != 0);
@@ -649,11 +654,9 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
         A.prop_w += within;
         A.prop_end += end;
         A.prop_b += birth;
-        A.prop_d += death;
         const bool proposed = within || born || (death && n > 2);
         const int jj = within ? jw : jd, kk = k;
         const int n_new = birth ? n + 1 : (death ? n - 1 : n);
-        const int inew = within ? jw : (birth ? k + 1 : -1);
         const int nc = (end || death) ? 2 : 3;
         const int onc = (end || birth) ? 2 : 3;
         const float3 fnew = within ? (end ? fend : fin) : (birth ? fbirth : f3(0.f, 0.f, 0.f));
@@ -743,7 +746,7 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
           A.acc_e += (move == MV_END);
           A.acc_b += (move == MV_BIRTH);
           A.acc_d += (move == MV_DEATH);
-          lane_close<kGrad>(A, t, R.burn_in, n, L, G);
+          lane_close<kGrad>(A, s, burn_in, n, L, G);
           if (move >= MV_BIRTH) {
             // a birth moves entries k+1 .. n-1 up by one (highest first), a death
             // entries j+1 .. n-1 down by one (lowest first); segment arrays only
@@ -846,15 +849,20 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
 #pragma unroll kRoll
               for (int i = max(a0, W); i <= n - 1; ++i) move_any(i, i - 1);
           }
-#pragma unroll
-          for (int v = 0; v < 3; ++v) {
-            if (v < nc) {
-              w.st(AVT, wlo + v, nvt[v]);
-              if constexpr (kGrad) w.st(AGT, wlo + v, ngt[v]);
-              if (v < nc - 1 && v < 2) w.set_segment(wlo + v, make_float2(nseg[v], nlen[v]));
-            }
+          // the new vertex is entry wlo + 1
+          w.st(AVT, wlo, nvt[0]);
+          if (death) w.st(AVT, wlo + 1, nvt[1]);
+          else w.set_vertex(wlo + 1, make_float4(fnew.x, fnew.y, fnew.z, nvt[1]));
+          w.set_segment(wlo, make_float2(nseg[0], nlen[0]));
+          if (three) {
+            w.st(AVT, wlo + 2, nvt[2]);
+            w.set_segment(wlo + 1, make_float2(nseg[1], nlen[1]));
           }
-          if (move != MV_DEATH) w.set_pos(inew, fnew);
+          if constexpr (kGrad) {
+#pragma unroll
+            for (int v = 0; v < 3; ++v)
+              if (v < nc) w.st(AGT, wlo + v, ngt[v]);
+          }
           n = n_new;
           L += dlen;
           G += dG;
@@ -888,7 +896,7 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
           taken = logu_mine < gain - lpo;
           if (taken) {
             A.acc_i++;
-            lane_close<kGrad>(A, t, R.burn_in, n, L, G);
+            lane_close<kGrad>(A, s, burn_in, n, L, G);
           }
         }
         if (__any_sync(kAll, taken)) {
@@ -905,7 +913,7 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
     if (((s + 1) & (kRefresh - 1)) == 0) lane_refresh_sums<kGrad>(w, n, L, G);
   }
   if (!own) return;
-  lane_close<kGrad>(A, step0 + done, R.burn_in, n, L, G);
+  lane_close<kGrad>(A, done, burn_in, n, L, G);
   lane_flush<kGrad>(A, acc);
   // recorded states, proposal and acceptance counts
   const unsigned long long t_end = step0 + done;
@@ -914,7 +922,7 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
   acc[ACC_PROP + 0] += static_cast<double>(A.prop_w - A.prop_end);
   acc[ACC_PROP + 1] += static_cast<double>(A.prop_end);
   acc[ACC_PROP + 2] += static_cast<double>(A.prop_b);
-  acc[ACC_PROP + 3] += static_cast<double>(A.prop_d);
+  acc[ACC_PROP + 3] += static_cast<double>(done - A.prop_w - A.prop_b);
   acc[ACC_ACC + 0] += static_cast<double>(A.acc_i);
   acc[ACC_ACC + 1] += static_cast<double>(A.acc_e);
   acc[ACC_ACC + 2] += static_cast<double>(A.acc_b);
