@@ -570,21 +570,37 @@ __device__ __forceinline__ void run_chain(const ChainParams& P, int c, bool own,
         const float target =
             __fmaf_rn(static_cast<float>(v23), 1.1920928955078125e-7f, 5.9604644775390625e-8f) * total;
         // (the cumulative sums rise with q: k counts those at or below u T_b,
-        // at most n - 2; no early exit, so the loads and sums pipeline)
+        // at most n - 2)
         int k = n - 2;
         if (born) {
           float cum = 0.f;
-          int below = 0;
+          int below = 0, q = 0;
+          bool over = false;
           const int m = min(n - 1, W);
-#pragma unroll 4
-          for (int q = 0; q < m; ++q) {
-            cum += M.b * *w.at(ALEN, q);
-            below += (cum <= target) ? 1 : 0;
+          // four segments per pass, ended by the first whose last sum exceeds the target
+#pragma unroll 1
+          for (; q + 4 <= m; q += 4) {
+            const float c0 = cum + M.b * *w.at(ALEN, q), c1 = c0 + M.b * *w.at(ALEN, q + 1);
+            const float c2 = c1 + M.b * *w.at(ALEN, q + 2), c3 = c2 + M.b * *w.at(ALEN, q + 3);
+            if (!(c3 <= target)) {
+              below = q + (c0 <= target) + (c1 <= target) + (c2 <= target);
+              over = true;
+              break;
+            }
+            cum = c3;
           }
-#pragma unroll kRoll
-          for (int q = W; q < n - 1; ++q) {
-            cum += M.b * w.gm[ALEN * cap + q];
-            below += (cum <= target) ? 1 : 0;
+          if (!over) {
+            below = q;
+#pragma unroll 1
+            for (; q < m; ++q) {
+              cum += M.b * *w.at(ALEN, q);
+              below += (cum <= target) ? 1 : 0;
+            }
+#pragma unroll 1
+            for (q = W; q < n - 1; ++q) {
+              cum += M.b * w.gm[ALEN * cap + q];
+              below += (cum <= target) ? 1 : 0;
+            }
           }
           k = min(below, n - 2);
         }
