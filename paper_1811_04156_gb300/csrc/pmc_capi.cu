@@ -176,6 +176,7 @@ struct ChainClass {
   int smem_cap = 0;   // shared window (vertices per chain)
   int max_cap = 0;    // largest vertex cap of the class's chains
   bool spill = false; // smem_cap < max_cap: entries beyond the window live in global memory
+  bool fuse_z = false; // rounding of a birth's z (birth_point)
   int lo = 0, hi = 0;  // range into the processing order
   int warps_per_block = 4;
   int grid = 0;
@@ -651,8 +652,7 @@ static ChainParams class_params(pmc_chains_t ch, size_t k, unsigned long long n_
   p.chain_hi = cl.hi;
   p.n_steps = n_steps;
   p.smem_cap = cl.smem_cap;
-  // a chain's results do not depend on the shared window: the cap alone sets the rounding
-  p.birth_fuse_z = cl.max_cap > 256;
+  p.birth_fuse_z = cl.fuse_z;
   return p;
 }
 
@@ -662,7 +662,8 @@ static ChainParams class_params(pmc_chains_t ch, size_t k, unsigned long long n_
 // code without spill tests, a quarter fewer instructions, and the probes of
 // the autotuner cannot see how long paths grow: 67,000 chains of 55-110
 // vertices (caps of 64 to 1,024) ran 1,000 steps in 39.1 ms with windows of
-// 128, 36.3 with 192, 30.8 with 256, 29.8 with 320.
+// 128, 36.3 with 192, 30.8 with 256, 29.8 with 320 (28.2 since the kernels
+// flush subnormals).
 static int warp_window(pmc_chains_t ch, int full) {
   int most = 0;
   if (chain_occupancy(ch->general, 0, ch->grad, full > 32, 4, 32, &most) != cudaSuccess) return full;
@@ -681,7 +682,7 @@ static int warp_window(pmc_chains_t ch, int full) {
 // whose paths are expected to stay within the groups' window (the straight
 // line's vertex count); 30,720 chains of 44 vertices in 100 layers, 500 steps:
 // 10.3 ms with one warp per chain (window 256), 6.9 ms in groups (window 128;
-// 8.4 with 96, 9.3 with 192).  The lean kernel's longer paths spill there
+// 8.4 with 96, 9.3 with 192; 6.2 flushing subnormals).  The lean kernel's longer paths spill there
 // (40 against 30 ms).  Teams: offered to the autotuner up to four chains per SM
 // (one warp per scheduler); 1,000 plain steps of 64 chains 0.94 ms with one warp
 // per chain, 0.75 with teams, of 608 chains 0.96 and 0.93, of 912 1.01 and 1.57
@@ -690,8 +691,8 @@ constexpr int kGroupChains = 20, kGroupWindow = 128, kTeamChains = 4;
 
 // Autotuner: for every cap class, time the chain kernel over candidate launch
 // shapes — 1, 2 or 4 warps per block; with one warp per chain the shared
-// window of warp_window (entries beyond it in global memory), four steps of a
-// chain per warp where the chains are few, or groups of 8 lanes per chain (rules
+// window of warp_window (entries beyond it in global memory), a team of four
+// warps per chain where the chains are few, or groups of 8 lanes per chain (rules
 // above); with one lane per chain (lean runs with short paths) a
 // per-lane window of 8 to 32 vertices — on a scratch copy of the freshly initialised
 // state (256 steps, best of two probes), and keep the fastest; choices are
@@ -1048,6 +1049,10 @@ int pmc_init_chains(pmc_ctx_t ctx, pmc_medium_t med, pmc_geom_t geom, const pmc_
   // initial paths exist), persistent grid from occupancy
   ch->autotune = r->warps_per_block <= 0 && r->smem_window <= 0;
   for (auto& cl : ch->classes) {
+    // tuned shapes: results do not depend on the window that the rule or the
+    // probes choose, the class's cap alone sets the rounding; shapes that the
+    // caller sets: the window does
+    cl.fuse_z = ch->autotune ? cl.max_cap > 256 : cl.spill;
     int wpb = r->warps_per_block > 0 ? r->warps_per_block : 4;
     wpb = std::min(wpb, 4);
     while (wpb > 1 && chain_smem_bytes(cl.smem_cap, wpb, cl.kind, cl.share, ch->grad) > ctx->smem_per_block) wpb /= 2;
