@@ -73,7 +73,8 @@ extern "C" {
 
 /* Chain layout of the kernel (pmc_run_desc.layout). */
 #define PMC_LAYOUT_AUTO 0      /* autotuner's choice (warp layout when warps_per_block is given) */
-#define PMC_LAYOUT_WARP 1      /* one warp per chain */
+#define PMC_LAYOUT_WARP 1      /* one warp per chain; left to the autotuner (warps_per_block = 0), also
+                                  8 lanes of a warp per chain or four warps per chain: the same chains */
 #define PMC_LAYOUT_LANE 2      /* one lane per chain: lean physics only (homogeneous medium, isotropic
                                   emission, rho = 1, pure Henyey-Greenstein) with Gaussian, MALA or
                                   tree moves */
@@ -400,7 +401,8 @@ PMC_API int pmc_total_chains(pmc_chains_t chains);
  * class's caps when entries beyond it live in global memory), first and
  * one-past-last position in the processing order, warps per block,
  * persistent grid size, and the kernel: 0 the lean and 1 the general kernel
- * with one warp per chain, 2 the general kernel with tree moves, 3 with HMC
+ * with one warp per chain (or what the autotuner took in its place: 8 lanes of
+ * a warp per chain, or the four warps of a block per chain), 2 the general kernel with tree moves, 3 with HMC
  * moves, 4 the lean kernel with one chain per lane (32 chains per warp), 5
  * the same with MALA moves, 6 the general kernel sampling the wavelength, 7
  * the lean kernel with tree moves, 8 the lean kernel with one chain per lane

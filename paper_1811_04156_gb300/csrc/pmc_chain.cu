@@ -1,4 +1,5 @@
-// Persistent RJMCMC chain kernel: one warp per chain, the chain's path staged
+// Persistent RJMCMC chain kernel: one warp per chain (a team of four warps
+// where the chains are few), the chain's path staged
 // in shared memory as SoA arrays with per-segment and per-vertex caches of the
 // log-density factors (Collin, arXiv:1811.04156: section "Numerical path
 // integration", Eq. acceptFact; appendix "Jump proposal" and "Dimension
@@ -27,8 +28,9 @@
 // 10 stall cycles per issue), since a step's code is longer than the
 // instruction cache serves to warps in different phases.  Loops over a path
 // are therefore kept rolled (`#pragma unroll 1`): 100 layers, 30,720 chains x
-// 500 steps 14.9 -> 13.4 ms; two-sensor tree moves, 4,096 chains x 200 steps
-// 5.3 -> 4.1 ms.
+// 500 steps 14.9 -> 13.4 ms (now 6.2 in groups of lanes, pmc_group.cuh);
+// two-sensor tree moves, 4,096 chains x 200 steps 5.3 -> 4.1 ms (3.7 flushing
+// subnormals).
 // kTree adds the paper's within-dimension move in tree coordinates (section
 // "Path proposal distribution"; appendix "Path space coordinate system"): the
 // whole path is re-expressed node by node in recursive bispherical systems,

@@ -8,12 +8,14 @@
 // would take it, each lane standing in for 32 / kG of them.
 //
 // Why: one warp per chain issues the proposal's scalar arithmetic, the change of
-// the log density (3 lanes busy) and the acceptance for 32 lanes, 406 warp
-// instructions per proposal, at 81 % of the issue slots.  With kG = 8, four
+// the log density (3 lanes busy) and the acceptance for 32 lanes, some 400 warp
+// instructions per proposal, at 58 to 81 % of the issue slots.  With kG = 8, four
 // chains share those instructions; only the O(n) parts (sums and shifts) take
 // more trips per chain.  The four chains draw different kinds of moves, so a
 // step runs as straight-line code with each kind's part behind a vote of the
-// warp rather than as four branches in turn.
+// warp rather than as four branches in turn.  30,720 chains of 44 vertices in
+// 100 layers, 500 steps: 10.3 ms with one warp per chain, 6.9 in groups (6.2
+// flushing subnormals).
 #pragma once
 
 #include <type_traits>

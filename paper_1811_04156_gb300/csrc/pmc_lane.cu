@@ -24,12 +24,14 @@
 // back to the global block at the start and end of a residency; the cached
 // factors are rebuilt at the start.
 //
-// Bound by instruction issue (64 % of the slots with 3.4 warps per scheduler).
-// The float4 / float2 layout and the branch-free factors took the detector run
-// (65,536 chains, mean n 11) from 47.7 to 43.6 warp instructions per proposal:
-// 4,000 steps with the estimate 18.6 -> 16.1 ms (float arrays and branching
-// factors -> branch-free 17.4 -> vectors 16.1); the MALA gradients run 17.5 ->
-// 16.9 ms.
+// Bound by instruction issue and, with 3.4 warps per scheduler, by the latency
+// of a step's dependent arithmetic.  65,536 chains of 11 vertices, 4,000 steps
+// with the estimate: 18.6 ms with float arrays and branching factors, 17.4 with
+// branch-free factors, 16.1 with the float4 / float2 layout (47.7 -> 43.6 warp
+// instructions per proposal), 14.6 flushing subnormals, 14.2 with 32-bit step
+// counts, 13.85 with the birth's search ended where it is found; 65,536 MALA
+// chains, 2,000 steps with scores 17.5 -> 15.7 ms.  (Moving the shorter side of
+// the path at births and deaths, entry 0 at a slot of its own per chain: 14.0.)
 #include "pmc_internal.h"
 #include "pmc_tree.cuh"
 
