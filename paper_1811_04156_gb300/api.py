@@ -338,9 +338,9 @@ class Chains:
 
     def read_states(self, stream=None):
         stride = self.geom.max_cap
-        xyz = np.zeros((self.total, 3, stride), dtype=np.float32)
-        n = np.zeros(self.total, dtype=np.int32)
-        steps = np.zeros(self.total, dtype=np.uint64)
+        xyz = np.empty((self.total, 3, stride), dtype=np.float32)
+        n = np.empty(self.total, dtype=np.int32)
+        steps = np.empty(self.total, dtype=np.uint64)
         check(load().pmc_read_states(self.handle, xyz.ctypes.data_as(C.POINTER(C.c_float)),
                                      n.ctypes.data_as(C.POINTER(C.c_int)),
                                      steps.ctypes.data_as(C.POINTER(C.c_uint64)), stride, _stream(stream)),
@@ -357,7 +357,8 @@ class Chains:
         return [dict(zip(keys, map(int, r))) for r in rows[: nc.value]]
 
     def read_accumulators(self, stream=None):
-        out = np.zeros((self.total, PMC_ACC_WORDS))
+        # the call writes every word: zeroing 8 MB first took longer than copying them (213 -> 72 us)
+        out = np.empty((self.total, PMC_ACC_WORDS))
         check(load().pmc_read_accumulators(self.handle, out.ctypes.data_as(C.POINTER(C.c_double)), out.size,
                                            _stream(stream)), "pmc_read_accumulators")
         return out
