@@ -1,6 +1,7 @@
 // C ABI of libpathmc (declared in include/pathmc.h): handle management,
 // validation, device buffers, CUDA-graph replay of the chain launches.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstring>
 #include <limits>
@@ -94,7 +95,7 @@ struct pmc_ctx_s {
   int n_sm = 0;
   size_t smem_per_sm = 0, smem_per_block = 0;
   // autotuned warps per block, keyed by (kernel instantiation, shared vertex cap, chain-count bucket)
-  std::map<std::tuple<int, int, int>, std::tuple<int, int, int, int>> tuned;  // -> (warps per block, window, kind, share)
+  std::map<std::tuple<int, int, int>, std::tuple<int, int, int, int, bool>> tuned;  // -> (warps per block, window, kind, share)
 };
 
 struct pmc_medium_s {
@@ -675,6 +676,26 @@ static int warp_window(pmc_chains_t ch, int full) {
   return std::min(full, 32);
 }
 
+// Rounding of a birth's z in tuned lean runs (birth_point): once (fused) where
+// a 128-vertex window would run the class in fewer waves of resident warps than
+// whole caps would, else twice.  That is where the instance with a window has
+// been the faster one, and the two instances round differently; a class keeps
+// its rounding whatever window it is tuned to now.
+static bool fused_births(pmc_chains_t ch, int full, int chains) {
+  if (ch->general != 0 || full <= 128) return false;
+  auto waves = [&](bool spill, int window) {
+    int most = 0;
+    for (int wpb : {1, 2, 4}) {
+      int bps = 0;
+      if (chain_smem_bytes(window, wpb, 0, 0, ch->grad) <= ch->ctx->smem_per_block &&
+          chain_occupancy(0, 0, ch->grad, spill, wpb, window, &bps) == cudaSuccess)
+        most = std::max(most, bps * wpb);
+    }
+    return most > 0 ? (chains + most * ch->ctx->n_sm - 1) / (most * ch->ctx->n_sm) : INT_MAX;
+  };
+  return waves(true, 128) < waves(false, full);
+}
+
 // When several chains share a warp, or a team of warps works on one.
 // Groups: the general physics with more chains than warps fit (20 per SM; 2,400
 // chains 0.98 ms with one warp per chain and 1.28 in groups, 3,600 1.74 and 1.39),
@@ -732,10 +753,11 @@ static int autotune_classes(pmc_chains_t ch, cudaStream_t s) {
     const int full = (cl.max_cap + 31) / 32 * 32;
     const auto key = std::make_tuple(kind_of(cl), cl.max_cap, bucket_of(chains));
     auto it = ch->ctx->tuned.find(key);
-    std::tuple<int, int, int, int> best(cl.warps_per_block, cl.smem_cap, cl.kind, cl.share);
+    std::tuple<int, int, int, int, bool> best(cl.warps_per_block, cl.smem_cap, cl.kind, cl.share, cl.fuse_z);
     if (it != ch->ctx->tuned.end()) {
       best = it->second;
     } else {
+      cl.fuse_z = fused_births(ch, full, chains);
       float best_ms = 1e30f;
       struct LaneProbe {
         float ms;
@@ -805,7 +827,7 @@ static int autotune_classes(pmc_chains_t ch, cudaStream_t s) {
           }
           if (ms < best_ms) {
             best_ms = ms;
-            best = std::make_tuple(wpb, win, ckind, share);
+            best = std::make_tuple(wpb, win, ckind, share, cl.fuse_z);
           }
           if (lane_kind(ckind))
             lane_probes.push_back({ms, wpb, win, ckind, (work_items(ckind, share, chains) + wpb - 1) / wpb <= grid});
@@ -826,10 +848,11 @@ static int autotune_classes(pmc_chains_t ch, cudaStream_t s) {
           if (!keep || std::make_tuple(pr.resident, pr.win, -pr.ms) > std::make_tuple(keep->resident, keep->win, -keep->ms))
             keep = &pr;
         }
-        if (keep) best = std::make_tuple(keep->wpb, keep->win, keep->kind, 0);
+        if (keep) best = std::make_tuple(keep->wpb, keep->win, keep->kind, 0, cl.fuse_z);
       }
       if (rc == PMC_OK) ch->ctx->tuned[key] = best;
     }
+    cl.fuse_z = std::get<4>(best);
     int bps = 0;
     const int bw = std::get<0>(best), bwin = std::get<1>(best), bkind = std::get<2>(best), bshare = std::get<3>(best);
     const bool spill = !lane_kind(bkind) && bwin < full;
@@ -1048,10 +1071,7 @@ int pmc_init_chains(pmc_ctx_t ctx, pmc_medium_t med, pmc_geom_t geom, const pmc_
   // initial paths exist), persistent grid from occupancy
   ch->autotune = r->warps_per_block <= 0 && r->smem_window <= 0;
   for (auto& cl : ch->classes) {
-    // tuned shapes: results do not depend on the window that the rule or the
-    // probes choose, the class's cap alone sets the rounding; shapes that the
-    // caller sets: the window does
-    cl.fuse_z = ch->autotune ? cl.max_cap > 256 : cl.spill;
+    cl.fuse_z = cl.spill;  // (tuned shapes: fused_births)
     int wpb = r->warps_per_block > 0 ? r->warps_per_block : 4;
     wpb = std::min(wpb, 4);
     while (wpb > 1 && chain_smem_bytes(cl.smem_cap, wpb, cl.kind, cl.share, ch->grad) > ctx->smem_per_block) wpb /= 2;

@@ -69,3 +69,18 @@ def test_teams_match_one_warp_per_chain(name):
     sc.run = dataclasses.replace(sc.run, burn_in=50, layout=S.LAYOUT_WARP)
     steps = (1500, 33, 1)
     _same(_run(sc, steps), _run(sc, steps, warps_per_block=2), 1)
+
+
+@pytest.mark.parametrize("chains,window", [(90, 0), (13, 0), (17, 128)])
+def test_tuned_long_caps_match_a_caller_set_shape(chains, window):
+    """Long vertex caps of lean runs: tuned chains are those of the whole cap in
+    shared memory while as many waves of warps hold them as with a window of
+    128, else those of the window (per SM: 16 warps of 512 vertices, 24 of 128)."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    sc = S.plain(n_chains=chains if chains > 64 else chains * n_sm, n_steps=1500, cap=512)
+    sc.run.layout = S.LAYOUT_WARP
+    a = _run(sc, (1500,))
+    _same(a, _run(sc, (1500,), warps_per_block=2, smem_window=window), ran=80)
