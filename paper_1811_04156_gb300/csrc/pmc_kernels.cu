@@ -44,11 +44,14 @@ constexpr int kTilePaths = 32;      // paths of a tile, and of a small batch's o
 constexpr int kTilePathsFew = 4;
 
 // Tiles of 4 paths (a warp each for their sums) where 32 would leave fewer than
-// three blocks per SM (paths of 21 vertices: 5,000 3.75 us in tiles of 4 and
+// three blocks per SM, eight where paths are longer than 64 (paths of 21 vertices: 5,000 3.75 us in tiles of 4 and
 // 6.69 in tiles of 32, 12,000 6.34 and 7.30, 14,500 7.07 and 7.40; 8,000 of 65
-// vertices 8.4 and 17.4), or where paths are long (the sums over more than 128
+// vertices 8.4 and 17.4, 14,700 12.3 and 17.8, 30,000 21.2 and 25.6, 65,536 as
+// fast in either), or where paths are long (the sums over more than 128
 // terms keep a warp's 32 partial sums).
-inline bool tile_few(int batch, int cap, int n_sm) { return cap > 128 || batch < 3 * kTilePaths * n_sm; }
+inline bool tile_few(int batch, int cap, int n_sm) {
+  return cap > 128 || batch < (cap > 64 ? 8 : 3) * kTilePaths * n_sm;
+}
 
 // First item of each of the tile's paths (invalid vertex counts: no items),
 // in offs[0 .. kP]; returns the number of items.
