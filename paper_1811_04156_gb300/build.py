@@ -29,13 +29,12 @@ NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompil
               "-I", INCLUDE] + ARCH
 
 
-# The chain kernels flush subnormal numbers: their approximate logarithms, roots
-# and divisions otherwise rescale subnormal arguments, two to three instructions
-# for each of the 20 to 30 per proposal.  Only lengths below 1e-19 m could
-# tell (the density enters as logarithms); the caller-facing density kernels
-# keep subnormals.  Detector run 16.0 -> 14.6 ms, two-sensor tree moves 4.16 ->
-# 3.67 ms, batched pairs 29.9 -> 28.2 ms, the same chains bit for bit.
-FTZ_SOURCES = ("pmc_chain.cu", "pmc_group.cu", "pmc_lane.cu")
+# The chain kernels are built twice: as they are, and with subnormals flushed,
+# for scenes in which no subnormal can arise (flush_is_exact in pmc_capi.cu);
+# their approximate logarithms, roots and divisions otherwise rescale subnormal
+# arguments, two to three instructions for each of the 20 to 30 per proposal.
+FLUSH_SOURCES = ("pmc_chain.cu", "pmc_group.cu", "pmc_lane.cu")
+FLUSH_FLAGS = ["-ftz=true", "-DPMC_FLUSH_SUBNORMALS"]
 
 
 def _nvcc() -> str:
@@ -94,17 +93,20 @@ def _build_locked(force: bool, verbose: bool, ptxas_info: bool) -> str:
     nvcc = _nvcc()
     extra = ["-Xptxas", "-v"] if ptxas_info else []
 
-    def compile_one(src):
-        obj = os.path.join(BUILD, os.path.basename(src) + ".o")
-        ftz = ["-ftz=true"] if os.path.basename(src) in FTZ_SOURCES else []
-        cmd = [nvcc, "-c", src, "-o", obj] + NVCC_FLAGS + ftz + extra
+    units = [(src, "", []) for src in _sources()]
+    units += [(src, ".flush", FLUSH_FLAGS) for src in _sources() if os.path.basename(src) in FLUSH_SOURCES]
+
+    def compile_one(unit):
+        src, variant, flags = unit
+        obj = os.path.join(BUILD, os.path.basename(src) + variant + ".o")
+        cmd = [nvcc, "-c", src, "-o", obj] + NVCC_FLAGS + flags + extra
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed for {src}:\n{r.stdout}\n{r.stderr}")
         return obj, r.stderr
 
     with cf.ThreadPoolExecutor(max_workers=min(8, os.cpu_count() or 1)) as ex:
-        results = list(ex.map(compile_one, _sources()))
+        results = list(ex.map(compile_one, units))
     if verbose or ptxas_info:
         for _, log in results:
             if log:

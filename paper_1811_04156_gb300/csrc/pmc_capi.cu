@@ -220,6 +220,7 @@ struct pmc_chains_s {
   cudaStream_t capture_stream = nullptr;
   std::vector<ChainClass> classes;
   std::map<unsigned long long, cudaGraphExec_t> graphs;
+  const ChainKernels* kernels = &full::kernels;  // or the kernels that flush subnormals (flush_is_exact)
   int general = 0;                 // chain kernel: 0 lean, 1 general, 2 with tree moves, 3 with HMC moves
   bool grad = false;               // keep d log sigma / dg per vertex
   bool autotune = false;           // warps per block chosen by timing
@@ -629,6 +630,46 @@ static int work_items(int kind, int share, int chains) {
   return (chains + per_item - 1) / per_item;
 }
 
+// Whether the chain kernels that flush subnormals step a scene exactly as the
+// others do (detector run 16.0 ms with subnormals, 14.6 without; two-sensor tree
+// moves 4.16, 3.67; batched pairs 29.9, 28.2).  The moves multiply up to four
+// lengths of a path (d1 d2 (d1 + d2) of an insertion; |e x rho|^2 against 1e-12
+// |e|^2 |rho|^2 in tree coordinates), and FP32 positions keep two vertices apart
+// by some 2^-24 of the scene.  From free paths and source-sensor distances of
+// 2^-8 m = 4 mm on, such products stay normal.  (Scenes of metres scaled
+// down by 2^10: the same chains bit for bit; by 2^20 one chain in 4,096 with tree
+// moves differs after 2,000 steps; by 2^40 most differ, with mean vertex counts
+// of 3.1 instead of 4.0.)  The other conditions keep products with b, the squares
+// of the sensor radius and of gradient steps, the weights of the phase mixture
+// and the spectrum in the normal range.  The rule looks at the whole geometry, so
+// that a window of chains runs as the whole set does.
+static bool flush_is_exact(const pmc_chains_s* ch, const pmc_run_desc* r) {
+  constexpr double kLeast = 1.0 / 256, kMost = 1099511627776.0;  // 2^-8, 2^40 m
+  constexpr double kTiny = 1.0 / 1073741824;                     // 2^-30
+  const pmc_medium_s* m = ch->med;
+  auto in_range = [&](double length) { return length >= kLeast && length <= kMost; };
+  if (m->d.kind != PMC_HOMOGENEOUS) {
+    for (double ls : m->ls_layers)
+      if (!in_range(ls)) return false;
+  } else if (!in_range(m->lambda_s)) {
+    return false;
+  }
+  for (const PairHost& h : ch->geom->host) {
+    double rel[3];
+    for (int i = 0; i < 3; ++i) rel[i] = h.c[i] - h.src[i];
+    if (!in_range(norm3(rel) - h.R) || !(h.R >= kTiny)) return false;
+  }
+  if (m->d.f_sl > 0.f && !(m->d.f_sl >= kTiny && m->d.f_sl < 1.f)) return false;
+  if ((r->within == PMC_WITHIN_MALA || r->within == PMC_WITHIN_HMC) && !(r->mala_step >= kTiny)) return false;
+  if (ch->lam_on) {
+    for (double lam : {ch->spec_x.front(), ch->spec_x.back()})
+      if (!in_range(m->lambda_s * std::pow(lam / m->d.lam0, m->d.ks))) return false;
+    for (double y : ch->spec_y)
+      if (y > 0.0 && !(y >= kTiny)) return false;
+  }
+  return true;
+}
+
 static ChainParams class_params(pmc_chains_t ch, size_t k, unsigned long long n_steps) {
   const ChainClass& cl = ch->classes[k];
   ChainParams p{};
@@ -666,11 +707,11 @@ static ChainParams class_params(pmc_chains_t ch, size_t k, unsigned long long n_
 // flush subnormals).
 static int warp_window(pmc_chains_t ch, int full) {
   int most = 0;
-  if (chain_occupancy(ch->general, 0, ch->grad, full > 32, 4, 32, &most) != cudaSuccess) return full;
+  if (ch->kernels->occupancy(ch->general, 0, ch->grad, full > 32, 4, 32, &most) != cudaSuccess) return full;
   for (int w = full; w > 32; w -= 32) {
     int bps = 0;
-    if (chain_smem_bytes(w, 4, ch->general, 0, ch->grad) <= ch->ctx->smem_per_block &&
-        chain_occupancy(ch->general, 0, ch->grad, w < full, 4, w, &bps) == cudaSuccess && bps >= most)
+    if (ch->kernels->smem_bytes(w, 4, ch->general, 0, ch->grad) <= ch->ctx->smem_per_block &&
+        ch->kernels->occupancy(ch->general, 0, ch->grad, w < full, 4, w, &bps) == cudaSuccess && bps >= most)
       return w;
   }
   return std::min(full, 32);
@@ -687,8 +728,8 @@ static bool fused_births(pmc_chains_t ch, int full, int chains) {
     int most = 0;
     for (int wpb : {1, 2, 4}) {
       int bps = 0;
-      if (chain_smem_bytes(window, wpb, 0, 0, ch->grad) <= ch->ctx->smem_per_block &&
-          chain_occupancy(0, 0, ch->grad, spill, wpb, window, &bps) == cudaSuccess)
+      if (ch->kernels->smem_bytes(window, wpb, 0, 0, ch->grad) <= ch->ctx->smem_per_block &&
+          ch->kernels->occupancy(0, 0, ch->grad, spill, wpb, window, &bps) == cudaSuccess)
         most = std::max(most, bps * wpb);
     }
     return most > 0 ? (chains + most * ch->ctx->n_sm - 1) / (most * ch->ctx->n_sm) : INT_MAX;
@@ -726,10 +767,10 @@ static int autotune_classes(pmc_chains_t ch, cudaStream_t s) {
   int* sstat = nullptr;
   float* slam = nullptr;  // wavelength sampling: the probes' copy of the wavelengths
   // cache key: the warp kernel instance, the layout request, which lane kernel
-  // (if any) the run may use and whether its vertex moves are Gaussian; per
-  // class also whether its paths are short and whether they fit a group's window
-  const int kind = ((((ch->general * 2 + ch->grad) * 3 + ch->layout) * 16 + ch->lane_kind) * 2 +
-                    (ch->run.within == PMC_WITHIN_PERTURB)) * 4;
+  // (if any) the run may use, whether its vertex moves are Gaussian and whether
+  // its kernels flush subnormals; per class also whether its paths are short and whether they fit a group's window
+  const int kind = (((((ch->general * 2 + ch->grad) * 3 + ch->layout) * 16 + ch->lane_kind) * 2 +
+                     (ch->run.within == PMC_WITHIN_PERTURB)) * 2 + (ch->kernels == &flush::kernels)) * 4;
   auto kind_of = [&](const ChainClass& cl) { return kind + cl.short_paths + 2 * (cl.expect_n <= kGroupWindow); };
   auto bucket_of = [](int chains) { return 31 - __builtin_clz(static_cast<unsigned>(std::max(1, chains))); };
   bool need = false;
@@ -787,9 +828,9 @@ static int autotune_classes(pmc_chains_t ch, cudaStream_t s) {
         for (int wpb : {1, 2, 4}) {
           if (share == kShareTeam && wpb != 4) continue;
           const bool spill = !lane_kind(ckind) && win < full;
-          if (chain_smem_bytes(win, wpb, ckind, share, ch->grad) > ch->ctx->smem_per_block) continue;
+          if (ch->kernels->smem_bytes(win, wpb, ckind, share, ch->grad) > ch->ctx->smem_per_block) continue;
           int bps = 0;
-          if (chain_occupancy(ckind, share, ch->grad, spill, wpb, win, &bps) != cudaSuccess || bps < 1) continue;
+          if (ch->kernels->occupancy(ckind, share, ch->grad, spill, wpb, win, &bps) != cudaSuccess || bps < 1) continue;
           const int grid = std::max(1, std::min((work_items(ckind, share, chains) + wpb - 1) / wpb, bps * ch->ctx->n_sm));
           ChainParams p = class_params(ch, k, 256);
           p.smem_cap = win;
@@ -814,7 +855,7 @@ static int autotune_classes(pmc_chains_t ch, cudaStream_t s) {
               e = cudaMemcpyAsync(slam, ch->d_lam, sizeof(float) * T, cudaMemcpyDeviceToDevice, s);
             if (e == cudaSuccess) e = cudaMemsetAsync(ch->d_queue + k, 0, sizeof(unsigned int), s);
             if (e == cudaSuccess) e = cudaEventRecord(e0, s);
-            if (e == cudaSuccess) e = launch_chain(p, ckind, share, ch->grad, spill, grid, wpb, s);
+            if (e == cudaSuccess) e = ch->kernels->launch(p, ckind, share, ch->grad, spill, grid, wpb, s);
             if (e == cudaSuccess) e = cudaEventRecord(e1, s);
             if (e == cudaSuccess) e = cudaEventSynchronize(e1);
             float t = 0.f;
@@ -856,7 +897,7 @@ static int autotune_classes(pmc_chains_t ch, cudaStream_t s) {
     int bps = 0;
     const int bw = std::get<0>(best), bwin = std::get<1>(best), bkind = std::get<2>(best), bshare = std::get<3>(best);
     const bool spill = !lane_kind(bkind) && bwin < full;
-    if (rc == PMC_OK && chain_occupancy(bkind, bshare, ch->grad, spill, bw, bwin, &bps) == cudaSuccess && bps >= 1) {
+    if (rc == PMC_OK && ch->kernels->occupancy(bkind, bshare, ch->grad, spill, bw, bwin, &bps) == cudaSuccess && bps >= 1) {
       cl.kind = bkind;
       cl.share = bshare;
       cl.warps_per_block = bw;
@@ -991,6 +1032,7 @@ int pmc_init_chains(pmc_ctx_t ctx, pmc_medium_t med, pmc_geom_t geom, const pmc_
   if (r->within == PMC_WITHIN_HMC) ch->general = 3;
   if (ch->lam_on) ch->general = 6;
   ch->layout = r->layout;
+  if (flush_is_exact(ch.get(), r)) ch->kernels = &flush::kernels;
   if (lean_physics && r->within == PMC_WITHIN_PERTURB && !ch->lam_on) ch->lane_kind = 4;
   if (lean_physics && r->within == PMC_WITHIN_MALA) ch->lane_kind = 5;
   if (lean_physics && r->within == PMC_WITHIN_TREE) ch->lane_kind = 8;
@@ -1074,10 +1116,10 @@ int pmc_init_chains(pmc_ctx_t ctx, pmc_medium_t med, pmc_geom_t geom, const pmc_
     cl.fuse_z = cl.spill;  // (tuned shapes: fused_births)
     int wpb = r->warps_per_block > 0 ? r->warps_per_block : 4;
     wpb = std::min(wpb, 4);
-    while (wpb > 1 && chain_smem_bytes(cl.smem_cap, wpb, cl.kind, cl.share, ch->grad) > ctx->smem_per_block) wpb /= 2;
-    if (chain_smem_bytes(cl.smem_cap, wpb, cl.kind, cl.share, ch->grad) > ctx->smem_per_block) return fail(PMC_ERR_INVALID, "vertex cap too large for shared memory");
+    while (wpb > 1 && ch->kernels->smem_bytes(cl.smem_cap, wpb, cl.kind, cl.share, ch->grad) > ctx->smem_per_block) wpb /= 2;
+    if (ch->kernels->smem_bytes(cl.smem_cap, wpb, cl.kind, cl.share, ch->grad) > ctx->smem_per_block) return fail(PMC_ERR_INVALID, "vertex cap too large for shared memory");
     int bps = 0;
-    CK(chain_occupancy(cl.kind, cl.share, ch->grad, cl.spill, wpb, cl.smem_cap, &bps));
+    CK(ch->kernels->occupancy(cl.kind, cl.share, ch->grad, cl.spill, wpb, cl.smem_cap, &bps));
     if (bps < 1) return fail(PMC_ERR_INVALID, "chain kernel does not fit on an SM");
     if (lane_kind(cl.kind) && r->warps_per_block <= 0) {
       // a lane-layout window set without warps per block: the shape that
@@ -1087,7 +1129,7 @@ int pmc_init_chains(pmc_ctx_t ctx, pmc_medium_t med, pmc_geom_t geom, const pmc_
       long best_res = static_cast<long>(std::min((items + wpb - 1) / wpb, bps * ctx->n_sm)) * wpb;
       for (int w2 = wpb / 2; w2 >= 1; w2 /= 2) {
         int b2 = 0;
-        CK(chain_occupancy(cl.kind, cl.share, ch->grad, cl.spill, w2, cl.smem_cap, &b2));
+        CK(ch->kernels->occupancy(cl.kind, cl.share, ch->grad, cl.spill, w2, cl.smem_cap, &b2));
         if (b2 < 1) continue;
         const long res = static_cast<long>(std::min((items + w2 - 1) / w2, b2 * ctx->n_sm)) * w2;
         if (res > best_res) {
@@ -1186,7 +1228,7 @@ int pmc_init_chains(pmc_ctx_t ctx, pmc_medium_t med, pmc_geom_t geom, const pmc_
     ip.user_n = d_user_n;
     ip.user_stride = r->init_stride;
   }
-  CK(launch_init(ip, s));
+  CK(ch->kernels->init(ip, s));
   // direct-sector integral per pair (axisymmetric integrands need one azimuth)
   const bool axisym = std::all_of(ch->h_pairs.begin(), ch->h_pairs.end(),
                                   [](const DPair& d) { return d.emission == 0 && d.rho == 0; }) &&
@@ -1264,7 +1306,7 @@ int pmc_reset_chains(pmc_chains_t ch, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   CK(cudaMemsetAsync(ch->d_status, 0, sizeof(int) * ch->total, s));
   CK(cudaMemsetAsync(ch->d_any, 0, sizeof(int), s));
-  CK(launch_init(init_params(ch), s));
+  CK(ch->kernels->init(init_params(ch), s));
   return PMC_OK;
 }
 
@@ -1293,7 +1335,7 @@ int pmc_set_states(pmc_chains_t ch, const float* xyz, const int* n, int stride, 
   ip.user_xyz = ch->d_stage;
   ip.user_n = ch->d_stage_n;
   ip.user_stride = stride;
-  CK(launch_init(ip, s));
+  CK(ch->kernels->init(ip, s));
   return PMC_OK;
 }
 
@@ -1306,7 +1348,7 @@ static int enqueue_steps(pmc_chains_t ch, unsigned long long n_steps, cudaStream
     for (unsigned long long left = n_steps; left > 0;) {
       const unsigned long long now = std::min(left, most);
       CK(cudaMemsetAsync(ch->d_queue + k, 0, sizeof(unsigned int), s));
-      CK(launch_chain(class_params(ch, k, now), cl.kind, cl.share, ch->grad, cl.spill, cl.grid, cl.warps_per_block, s));
+      CK(ch->kernels->launch(class_params(ch, k, now), cl.kind, cl.share, ch->grad, cl.spill, cl.grid, cl.warps_per_block, s));
       left -= now;
     }
   }

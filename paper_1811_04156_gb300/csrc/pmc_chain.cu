@@ -43,6 +43,7 @@
 #include "pmc_warp.cuh"
 
 namespace pmc {
+namespace PMC_VARIANT {
 
 namespace {
 
@@ -1070,10 +1071,6 @@ int kernel_key(int kind, int share, bool grad, bool spill) {
   return (kind == 1 ? 4 : 0) + (grad ? 2 : 0) + (spill ? 1 : 0);
 }
 
-}  // namespace
-
-int chain_arrays(bool general, bool grad) { return 6 + (general ? 1 : 0) + (grad ? 1 : 0); }
-
 size_t chain_smem_bytes(int smem_cap, int warps_per_block, int kind, int share, bool grad) {
   if (share == kShareGroup) return group_smem_bytes(grad, smem_cap, warps_per_block);
   if (share == kShareTeam)
@@ -1160,4 +1157,9 @@ cudaError_t launch_init(const InitParams& p, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+}  // namespace
+
+const ChainKernels kernels = {launch_chain, chain_smem_bytes, chain_occupancy, launch_init};
+
+}  // namespace PMC_VARIANT
 }  // namespace pmc

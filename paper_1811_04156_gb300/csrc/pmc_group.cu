@@ -3,6 +3,7 @@
 #include "pmc_group.cuh"
 
 namespace pmc {
+namespace PMC_VARIANT {
 
 size_t group_smem_bytes(bool grad, int smem_cap, int warps_per_block) {
   return static_cast<size_t>(warps_per_block) * (32 / kGroupLanes) *
@@ -20,4 +21,5 @@ cudaError_t group_kernel(bool grad, bool spill, const ChainParams* p, int grid, 
               : group_call<true, false, false, kG>(p, grid, warps_per_block, smem, blocks_per_sm, s);
 }
 
+}  // namespace PMC_VARIANT
 }  // namespace pmc

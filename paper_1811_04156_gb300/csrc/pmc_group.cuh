@@ -23,6 +23,7 @@
 #include "pmc_warp.cuh"
 
 namespace pmc {
+namespace PMC_VARIANT {
 
 namespace {
 
@@ -690,4 +691,5 @@ cudaError_t group_call(const ChainParams* p, int grid, int warps_per_block, size
 
 }  // namespace
 
+}  // namespace PMC_VARIANT
 }  // namespace pmc

@@ -93,12 +93,35 @@ constexpr int kLaneTreeArrays = 4;
 // same results.
 constexpr int kShareGroup = 1, kShareTeam = 2;
 constexpr int kGroupLanes = 8;
-int chain_arrays(bool general, bool grad);
-cudaError_t launch_chain(const ChainParams& p, int kind, int share, bool grad, bool spill, int grid,
-                         int warps_per_block, cudaStream_t s);
-size_t chain_smem_bytes(int smem_cap, int warps_per_block, int kind, int share, bool grad);
-cudaError_t chain_occupancy(int kind, int share, bool grad, bool spill, int warps_per_block, int smem_cap,
-                            int* blocks_per_sm);
+inline int chain_arrays(bool general, bool grad) { return 6 + (general ? 1 : 0) + (grad ? 1 : 0); }
+
+struct InitParams;
+struct ChainKernels {
+  cudaError_t (*launch)(const ChainParams& p, int kind, int share, bool grad, bool spill, int grid,
+                        int warps_per_block, cudaStream_t s);
+  size_t (*smem_bytes)(int smem_cap, int warps_per_block, int kind, int share, bool grad);
+  cudaError_t (*occupancy)(int kind, int share, bool grad, bool spill, int warps_per_block, int smem_cap,
+                           int* blocks_per_sm);
+  cudaError_t (*init)(const InitParams& p, cudaStream_t s);
+};
+
+// The chain kernels' sources (pmc_chain.cu, pmc_group.cu, pmc_lane.cu) are
+// built twice: as they are, and with subnormal results and arguments flushed to
+// zero (build.py, FLUSH_SOURCES), which drops the rescaling of subnormal
+// arguments around every approximate logarithm, root and division.
+#ifdef PMC_FLUSH_SUBNORMALS
+#define PMC_VARIANT flush
+#else
+#define PMC_VARIANT full
+#endif
+namespace full {
+extern const ChainKernels kernels;
+}
+namespace flush {
+extern const ChainKernels kernels;
+}
+
+namespace PMC_VARIANT {
 
 // pmc_group.cu: launch, or occupancy when blocks_per_sm is given.
 size_t group_smem_bytes(bool grad, int smem_cap, int warps_per_block);
@@ -111,6 +134,8 @@ size_t lane_smem_bytes(int window, int warps_per_block, bool grad, bool tree);
 cudaError_t lane_occupancy(int kind, int warps_per_block, int window, bool grad, int* blocks_per_sm);
 cudaError_t launch_lane_chain(const ChainParams& p, int kind, int grid, int warps_per_block, bool grad,
                               cudaStream_t s);
+
+}  // namespace PMC_VARIANT
 
 struct InitParams {
   DRun R;
@@ -131,7 +156,6 @@ struct InitParams {
   const int* user_n;
   int user_stride;
 };
-cudaError_t launch_init(const InitParams& p, cudaStream_t s);
 
 // pmc_kernels.cu
 cudaError_t launch_logp(const DMedium& M, const DPair& S, const float* xyz, const int* n, int batch, int cap,

@@ -36,6 +36,7 @@
 #include "pmc_tree.cuh"
 
 namespace pmc {
+namespace PMC_VARIANT {
 
 namespace {
 
@@ -1099,4 +1100,5 @@ cudaError_t launch_lane_chain(const ChainParams& p, int kind, int grid, int warp
               : launch_w<false, false, false>(p, grid, warps_per_block, s);
 }
 
+}  // namespace PMC_VARIANT
 }  // namespace pmc
