@@ -95,7 +95,7 @@ struct pmc_ctx_s {
   int n_sm = 0;
   size_t smem_per_sm = 0, smem_per_block = 0;
   // autotuned warps per block, keyed by (kernel instantiation, shared vertex cap, chain-count bucket)
-  std::map<std::tuple<int, int, int>, std::tuple<int, int, int, int, bool>> tuned;  // -> (warps per block, window, kind, share)
+  std::map<std::tuple<int, int, int>, std::tuple<int, int, int, int>> tuned;  // -> (warps per block, window, kind, share)
 };
 
 struct pmc_medium_s {
@@ -176,6 +176,7 @@ struct ChainClass {
   int expect_n = 0;   // vertices of the class's longest straight source-sensor line: 2 + its scattering depth
   int smem_cap = 0;   // shared window (vertices per chain)
   int max_cap = 0;    // largest vertex cap of the class's chains
+  int set_cap = 0, set_chains = 0;  // the same, and the number of chains, over the whole geometry
   bool spill = false; // smem_cap < max_cap: entries beyond the window live in global memory
   bool fuse_z = false; // rounding of a birth's z (birth_point)
   int lo = 0, hi = 0;  // range into the processing order
@@ -721,8 +722,11 @@ static int warp_window(pmc_chains_t ch, int full) {
 // a 128-vertex window would run the class in fewer waves of resident warps than
 // whole caps would, else twice.  That is where the instance with a window has
 // been the faster one, and the two instances round differently; a class keeps
-// its rounding whatever window it is tuned to now.
-static bool fused_births(pmc_chains_t ch, int full, int chains) {
+// its rounding whatever window it is tuned to now.  The rounding depends on the
+// geometry alone, not on the chain window or on what the context ran before:
+// a window's chains step as they do in the whole set.
+static bool fused_births(pmc_chains_t ch, const ChainClass& cl) {
+  const int full = (cl.set_cap + 31) / 32 * 32, chains = cl.set_chains;
   if (ch->general != 0 || full <= 128) return false;
   auto waves = [&](bool spill, int window) {
     int most = 0;
@@ -794,11 +798,10 @@ static int autotune_classes(pmc_chains_t ch, cudaStream_t s) {
     const int full = (cl.max_cap + 31) / 32 * 32;
     const auto key = std::make_tuple(kind_of(cl), cl.max_cap, bucket_of(chains));
     auto it = ch->ctx->tuned.find(key);
-    std::tuple<int, int, int, int, bool> best(cl.warps_per_block, cl.smem_cap, cl.kind, cl.share, cl.fuse_z);
+    std::tuple<int, int, int, int> best(cl.warps_per_block, cl.smem_cap, cl.kind, cl.share);
     if (it != ch->ctx->tuned.end()) {
       best = it->second;
     } else {
-      cl.fuse_z = fused_births(ch, full, chains);
       float best_ms = 1e30f;
       struct LaneProbe {
         float ms;
@@ -868,7 +871,7 @@ static int autotune_classes(pmc_chains_t ch, cudaStream_t s) {
           }
           if (ms < best_ms) {
             best_ms = ms;
-            best = std::make_tuple(wpb, win, ckind, share, cl.fuse_z);
+            best = std::make_tuple(wpb, win, ckind, share);
           }
           if (lane_kind(ckind))
             lane_probes.push_back({ms, wpb, win, ckind, (work_items(ckind, share, chains) + wpb - 1) / wpb <= grid});
@@ -889,11 +892,10 @@ static int autotune_classes(pmc_chains_t ch, cudaStream_t s) {
           if (!keep || std::make_tuple(pr.resident, pr.win, -pr.ms) > std::make_tuple(keep->resident, keep->win, -keep->ms))
             keep = &pr;
         }
-        if (keep) best = std::make_tuple(keep->wpb, keep->win, keep->kind, 0, cl.fuse_z);
+        if (keep) best = std::make_tuple(keep->wpb, keep->win, keep->kind, 0);
       }
       if (rc == PMC_OK) ch->ctx->tuned[key] = best;
     }
-    cl.fuse_z = std::get<4>(best);
     int bps = 0;
     const int bw = std::get<0>(best), bwin = std::get<1>(best), bkind = std::get<2>(best), bshare = std::get<3>(best);
     const bool spill = !lane_kind(bkind) && bwin < full;
@@ -1069,6 +1071,13 @@ int pmc_init_chains(pmc_ctx_t ctx, pmc_medium_t med, pmc_geom_t geom, const pmc_
     if (ka != kb) return ka < kb;
     return ca > cb;
   });
+  // every class over the whole geometry, whatever the chain window: largest cap, number of chains
+  std::map<int, std::pair<int, int>> set_classes;
+  for (const DPair& d : geom->pairs) {
+    auto& set = set_classes[class_key(d.cap)];
+    set.first = std::max(set.first, d.cap);
+    set.second += d.n_chains;
+  }
   for (int lo = 0; lo < T;) {
     const int k = class_key(ch->h_pairs[ch->h_pair_of[order[lo]]].cap);
     int hi = lo;
@@ -1092,6 +1101,7 @@ int pmc_init_chains(pmc_ctx_t ctx, pmc_medium_t med, pmc_geom_t geom, const pmc_
     cl.short_paths = med->d.kind == PMC_HOMOGENEOUS && max_n <= kLaneMaxN;
     cl.smem_cap = (maxcap + 31) / 32 * 32;
     cl.max_cap = maxcap;
+    std::tie(cl.set_cap, cl.set_chains) = set_classes[k];
     cl.expect_n = static_cast<int>(std::min(expect_n, 1e6));
     cl.spill = false;
     if (r->layout == PMC_LAYOUT_LANE) {
@@ -1113,7 +1123,9 @@ int pmc_init_chains(pmc_ctx_t ctx, pmc_medium_t med, pmc_geom_t geom, const pmc_
   // initial paths exist), persistent grid from occupancy
   ch->autotune = r->warps_per_block <= 0 && r->smem_window <= 0;
   for (auto& cl : ch->classes) {
-    cl.fuse_z = cl.spill;  // (tuned shapes: fused_births)
+    cl.fuse_z = ch->autotune ? fused_births(ch.get(), cl)
+                             : r->layout != PMC_LAYOUT_LANE && r->smem_window > 0 &&
+                                   r->smem_window < (cl.set_cap + 31) / 32 * 32;
     int wpb = r->warps_per_block > 0 ? r->warps_per_block : 4;
     wpb = std::min(wpb, 4);
     while (wpb > 1 && ch->kernels->smem_bytes(cl.smem_cap, wpb, cl.kind, cl.share, ch->grad) > ctx->smem_per_block) wpb /= 2;
