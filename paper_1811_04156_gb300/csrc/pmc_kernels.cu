@@ -47,8 +47,7 @@ constexpr int kTilePathsFew = 4;
 // three blocks per SM, eight where paths are longer than 64 (paths of 21 vertices: 5,000 3.75 us in tiles of 4 and
 // 6.69 in tiles of 32, 12,000 6.34 and 7.30, 14,500 7.07 and 7.40; 8,000 of 65
 // vertices 8.4 and 17.4, 14,700 12.3 and 17.8, 30,000 21.2 and 25.6, 65,536 as
-// fast in either), or where paths are long (the sums over more than 128
-// terms keep a warp's 32 partial sums).
+// fast in either), or where the cap exceeds 128 (tiles of 32 were not measured there).
 inline bool tile_few(int batch, int cap, int n_sm) {
   return cap > 128 || batch < (cap > 64 ? 8 : 3) * kTilePaths * n_sm;
 }
@@ -83,22 +82,45 @@ __device__ __forceinline__ int tile_path(const int* offs, int f) {
   return p;
 }
 
-// Sums over a chunk's items [c0, c1) of the path that this thread helps to
-// add up (kTile / kP threads per path, strided by the vertex index).
+// Sum of a chunk's items [c0, c1) of the path that this thread helps to add up
+// (kTile / kP threads per path): term i of the path goes to partial sum i mod 32
+// (mod 64 in tiles of 4 paths), and a thread's partial sums meet in pairs, then the
+// threads', as 32 lanes would add the path up.  So a path of at most 32 vertices
+// has the same log p whatever tile it is in.  (Eight partial sums per path in tiles of
+// 32 lost accuracy: 4.07e-8 from 64 bits on 131,072 paths of 21 vertices, against
+// 4.02e-8 with 32 at the same time, 31 us.)
 template <int kP>
 __device__ __forceinline__ float tile_partial(const int* offs, const float* term, int c0, int c1) {
-  constexpr int kT = kTile / kP;
+  constexpr int kT = kTile / kP, kA = kT < 32 ? 32 / kT : 2, kS = kT * kA;
   const int p = threadIdx.x / kT, part = threadIdx.x % kT;
   const int o = offs[p], hi = min(offs[p + 1], c1);
+  float v[kA];
+#pragma unroll
+  for (int j = 0; j < kA; ++j) v[j] = 0.f;
   int f = o + part;
-  if (f < c0) f += (c0 - f + kT - 1) / kT * kT;
-  float v = 0.f, u = 0.f;  // two sums: shorter chains of roundings
-  for (; f + kT < hi; f += 2 * kT) {
-    v += term[f - c0];
-    u += term[f + kT - c0];
+  if (o < c0) {  // the path began in an earlier chunk: its stride that holds c0
+    f += (c0 - o) / kS * kS;
+#pragma unroll
+    for (int j = 0; j < kA; ++j) {
+      const int q = f + j * kT;
+      if (q >= c0 && q < hi) v[j] += term[q - c0];
+    }
+    f += kS;
   }
-  if (f < hi) v += term[f - c0];
-  return v + u;
+  for (; f + (kA - 1) * kT < hi; f += kS) {
+#pragma unroll
+    for (int j = 0; j < kA; ++j) v[j] += term[f + j * kT - c0];
+  }
+#pragma unroll
+  for (int j = 0; j < kA - 1; ++j) {
+    if (f + j * kT >= hi) break;
+    v[j] += term[f + j * kT - c0];
+  }
+#pragma unroll
+  for (int h = kA / 2; h > 0; h >>= 1)
+#pragma unroll
+    for (int j = 0; j < h; ++j) v[j] += v[j + h];
+  return v[0];
 }
 template <int kP>
 __device__ __forceinline__ float tile_total(float v) {
