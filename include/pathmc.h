@@ -451,7 +451,8 @@ PMC_API int pmc_logp_grad(pmc_ctx_t ctx, pmc_medium_t medium, pmc_geom_t geom, i
                   const float* xyz, const int* n, int batch, int cap,
                   float* out_logp, float* out_grad, void* stream);
 
-/* d log p / d theta per path (async); out: device float32 [batch][n_theta]. */
+/* d log p / d theta per path (async); out: device float32 [batch][n_theta].
+ * A vertex count below 2 or above cap gives a row of zeros. */
 PMC_API int pmc_score(pmc_ctx_t ctx, pmc_medium_t medium, pmc_geom_t geom, int pair,
               const float* xyz, const int* n, int batch, int cap, float* out, void* stream);
 

@@ -278,7 +278,10 @@ __global__ void __launch_bounds__(128, 12) score_kernel(const DMedium M, const D
     __syncwarp();  // orders the zeros before the other lanes' additions
   }
   const int n = nn[b];
-  if (n < 2 || n > cap) return;
+  if (n < 2 || n > cap) {  // an invalid vertex count scores zero
+    if (M.kind == 0 && lane < n_theta) o[lane] = 0.f;
+    return;
+  }
   const float zoff = S.zoff;
   BatchPos pos{xyz, static_cast<size_t>(batch) * cap, static_cast<size_t>(b) * cap};
   if (M.kind == 0) {
