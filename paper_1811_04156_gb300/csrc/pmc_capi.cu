@@ -94,7 +94,7 @@ struct pmc_ctx_s {
   int device = 0;
   int n_sm = 0;
   size_t smem_per_sm = 0, smem_per_block = 0;
-  // autotuned warps per block, keyed by (kernel instantiation, shared vertex cap, chain-count bucket)
+  // autotuned shapes, keyed by (kernels and rules, largest cap, power of two of the chain count; autotune_classes)
   std::map<std::tuple<int, int, int>, std::tuple<int, int, int, int>> tuned;  // -> (warps per block, window, kind, share)
 };
 
@@ -753,6 +753,13 @@ static bool fused_births(pmc_chains_t ch, const ChainClass& cl) {
 // per chain, 0.75 with teams, of 608 chains 0.96 and 0.93, of 912 1.01 and 1.57
 // (100 layers: 1.39 and 1.16, 1.41 and 1.45, 1.49 and 2.55).
 constexpr int kGroupChains = 20, kGroupWindow = 128, kTeamChains = 4;
+static bool offers_teams(const pmc_chains_s* ch, const ChainClass& cl) {
+  return ch->general < 2 && cl.hi - cl.lo <= kTeamChains * ch->ctx->n_sm;
+}
+static bool takes_groups(const pmc_chains_s* ch, const ChainClass& cl) {
+  return ch->general == 1 && ch->run.within == PMC_WITHIN_PERTURB && cl.hi - cl.lo >= kGroupChains * ch->ctx->n_sm &&
+         cl.expect_n <= kGroupWindow;
+}
 
 // Autotuner: for every cap class, time the chain kernel over candidate launch
 // shapes — 1, 2 or 4 warps per block; with one warp per chain the shared
@@ -772,10 +779,14 @@ static int autotune_classes(pmc_chains_t ch, cudaStream_t s) {
   float* slam = nullptr;  // wavelength sampling: the probes' copy of the wavelengths
   // cache key: the warp kernel instance, the layout request, which lane kernel
   // (if any) the run may use, whether its vertex moves are Gaussian and whether
-  // its kernels flush subnormals; per class also whether its paths are short and whether they fit a group's window
+  // its kernels flush subnormals; per class its largest cap, the power of two of
+  // its chain count, and the outcome of each rule that decides its candidates
+  // (their limits lie between powers of two)
   const int kind = (((((ch->general * 2 + ch->grad) * 3 + ch->layout) * 16 + ch->lane_kind) * 2 +
-                     (ch->run.within == PMC_WITHIN_PERTURB)) * 2 + (ch->kernels == &flush::kernels)) * 4;
-  auto kind_of = [&](const ChainClass& cl) { return kind + cl.short_paths + 2 * (cl.expect_n <= kGroupWindow); };
+                     (ch->run.within == PMC_WITHIN_PERTURB)) * 2 + (ch->kernels == &flush::kernels)) * 8;
+  auto kind_of = [&](const ChainClass& cl) {
+    return kind + cl.short_paths + 2 * offers_teams(ch, cl) + 4 * takes_groups(ch, cl);
+  };
   auto bucket_of = [](int chains) { return 31 - __builtin_clz(static_cast<unsigned>(std::max(1, chains))); };
   bool need = false;
   for (auto& cl : ch->classes)
@@ -815,9 +826,8 @@ static int autotune_classes(pmc_chains_t ch, cudaStream_t s) {
       std::vector<std::tuple<int, int, int>> cands;
       if (ch->layout != PMC_LAYOUT_LANE) {
         cands.emplace_back(ch->general, ch->general < 2 ? warp_window(ch, full) : full, 0);
-        if (ch->general < 2 && chains <= kTeamChains * ch->ctx->n_sm) cands.emplace_back(ch->general, full, kShareTeam);
-        if (ch->general == 1 && ch->run.within == PMC_WITHIN_PERTURB && chains >= kGroupChains * ch->ctx->n_sm &&
-            cl.expect_n <= kGroupWindow)
+        if (offers_teams(ch, cl)) cands.emplace_back(ch->general, full, kShareTeam);
+        if (takes_groups(ch, cl))
           cands.assign(1, std::make_tuple(ch->general, std::min(full, kGroupWindow), kShareGroup));
       }
       if (ch->layout == PMC_LAYOUT_LANE ||

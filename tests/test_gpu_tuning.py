@@ -74,3 +74,33 @@ def test_windows_with_a_caller_set_window_replay_the_whole_set(n_sm):
     for lo in (0, 256):
         part = _run(api.Context(0), sc, 1500, chain_window=(lo, lo + 256), **shape)
         _same(part, [x[lo:lo + 256] for x in whole])
+
+
+def _is_team(row):
+    """A team of four warps per chain has a block per chain, one warp per chain a block per four."""
+    chains = row["hi"] - row["lo"]
+    return row["warps_per_block"] == 4 and row["grid"] > (chains + 3) // 4
+
+
+@pytest.mark.parametrize("per_sm", [(21, 15), (15, 21)])
+def test_groups_do_not_depend_on_earlier_sets(n_sm, per_sm):
+    """Chain counts of one power of two on both sides of the groups' 20 chains per SM."""
+    from paper_1811_04156_gb300 import api
+    ctx = api.Context(0)
+    for k in per_sm:
+        sc = S.general_small(n_chains=k * n_sm)
+        sc.pairs = [dataclasses.replace(sc.pairs[0], cap=200)]
+        assert _chains(ctx, sc).launch_info()[0]["smem_cap"] == (128 if k > 20 else 224)
+
+
+def test_no_team_for_many_chains_after_a_team_for_few(n_sm):
+    """The teams' limit, four chains per SM, lies between powers of two as well.  Near
+    it a probe may choose either, so in a few contexts."""
+    from paper_1811_04156_gb300 import api
+    for _ in range(8):
+        ctx = api.Context(0)
+        for chains in (7 * n_sm // 2, 5 * n_sm):
+            sc = S.plain(n_chains=chains)
+            sc.run.layout = S.LAYOUT_WARP
+            row = _chains(ctx, sc).launch_info()[0]
+        assert not _is_team(row), row
