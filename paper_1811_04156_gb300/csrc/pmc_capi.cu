@@ -700,15 +700,18 @@ static ChainParams class_params(pmc_chains_t ch, size_t k, unsigned long long n_
 
 // Window of the warp-per-chain kernels: the largest one that leaves the
 // number of resident warps to the registers (320 vertices for the lean kernel,
-// 288 or 256 for the general one).  Steps of paths that fit it take the kernel's
-// code without spill tests, a quarter fewer instructions, and the probes of
-// the autotuner cannot see how long paths grow: 67,000 chains of 55-110
-// vertices (caps of 64 to 1,024) ran 1,000 steps in 39.1 ms with windows of
-// 128, 36.3 with 192, 30.8 with 256, 29.8 with 320 (28.2 since the kernels
-// flush subnormals).
-static int warp_window(pmc_chains_t ch, int full) {
+// 352 or 288 for the general one) or to the chains there are.  Steps of paths
+// that fit it take the kernel's code without spill tests, a quarter fewer
+// instructions, and the probes of the autotuner cannot see how long paths grow:
+// 67,000 chains of 55-110 vertices (caps of 64 to 1,024) ran 1,000 steps in
+// 39.1 ms with windows of 128, 36.3 with 192, 30.8 with 256, 29.8 with 320 (28.2
+// since the kernels flush subnormals).  With few chains a larger window costs
+// nothing: 1,216 lean chains of 456 vertices (cap 1,024), 200 steps, 0.56 ms with
+// a window of 256, 0.29 with the whole cap.
+static int warp_window(pmc_chains_t ch, int full, int chains) {
   int most = 0;
   if (ch->kernels->occupancy(ch->general, 0, ch->grad, full > 32, 4, 32, &most) != cudaSuccess) return full;
+  most = std::min(most, (chains + 4 * ch->ctx->n_sm - 1) / (4 * ch->ctx->n_sm));
   for (int w = full; w > 32; w -= 32) {
     int bps = 0;
     if (ch->kernels->smem_bytes(w, 4, ch->general, 0, ch->grad) <= ch->ctx->smem_per_block &&
@@ -825,7 +828,7 @@ static int autotune_classes(pmc_chains_t ch, cudaStream_t s) {
       // windows of 8 to 32 vertices
       std::vector<std::tuple<int, int, int>> cands;
       if (ch->layout != PMC_LAYOUT_LANE) {
-        cands.emplace_back(ch->general, ch->general < 2 ? warp_window(ch, full) : full, 0);
+        cands.emplace_back(ch->general, ch->general < 2 ? warp_window(ch, full, chains) : full, 0);
         if (offers_teams(ch, cl)) cands.emplace_back(ch->general, full, kShareTeam);
         if (takes_groups(ch, cl))
           cands.assign(1, std::make_tuple(ch->general, std::min(full, kGroupWindow), kShareGroup));
@@ -907,7 +910,9 @@ static int autotune_classes(pmc_chains_t ch, cudaStream_t s) {
       if (rc == PMC_OK) ch->ctx->tuned[key] = best;
     }
     int bps = 0;
-    const int bw = std::get<0>(best), bwin = std::get<1>(best), bkind = std::get<2>(best), bshare = std::get<3>(best);
+    const int bw = std::get<0>(best), bkind = std::get<2>(best), bshare = std::get<3>(best);
+    // (the warp layout's window follows the number of chains, which the key holds coarsely)
+    const int bwin = bshare == 0 && bkind < 2 ? warp_window(ch, full, chains) : std::get<1>(best);
     const bool spill = !lane_kind(bkind) && bwin < full;
     if (rc == PMC_OK && ch->kernels->occupancy(bkind, bshare, ch->grad, spill, bw, bwin, &bps) == cudaSuccess && bps >= 1) {
       cl.kind = bkind;

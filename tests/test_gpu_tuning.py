@@ -104,3 +104,15 @@ def test_no_team_for_many_chains_after_a_team_for_few(n_sm):
             sc.run.layout = S.LAYOUT_WARP
             row = _chains(ctx, sc).launch_info()[0]
         assert not _is_team(row), row
+
+
+def test_the_window_follows_the_number_of_chains(n_sm):
+    """Eight warps per SM hold whole caps of 1,024 vertices, twelve do not; the counts are
+    of one power of two."""
+    from paper_1811_04156_gb300 import api
+    ctx = api.Context(0)
+    for per_sm in (12, 8, 12):
+        sc = S.plain(n_chains=per_sm * n_sm, cap=1024)
+        sc.run.layout = S.LAYOUT_WARP
+        window = _chains(ctx, sc).launch_info()[0]["smem_cap"]
+        assert window == 1024 if per_sm == 8 else 320 <= window < 1024, (per_sm, window)
