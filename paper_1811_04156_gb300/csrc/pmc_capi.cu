@@ -169,6 +169,13 @@ struct pmc_geom_s {
   int max_cap = 0;
 };
 
+// Launch shape of one chain kernel (ChainClass below).
+struct LaunchShape {
+  int share;
+  bool spill;
+  int smem_cap, warps_per_block, grid;
+};
+
 struct ChainClass {
   int kind = 0;       // kernel kind of launch_chain (4: one lane per chain)
   int share = 0;      // kinds 0 and 1: how a warp's lanes share its chains (kShareGroup, kShareTeam)
@@ -182,6 +189,9 @@ struct ChainClass {
   int lo = 0, hi = 0;  // range into the processing order
   int warps_per_block = 4;
   int grid = 0;
+  std::vector<LaunchShape> others;  // kernels that may run in this one's place, by the paths of the moment
+  ChoiceRule rule{};
+  bool grows = false;  // paths of the geometry are expected to grow long: long runs are cut
 };
 
 struct pmc_chains_s {
@@ -208,6 +218,7 @@ struct pmc_chains_s {
   int* d_status = nullptr;
   int* d_any = nullptr;  // OR of the status words, in the word after d_est (one copy reads both)
   unsigned int* d_queue = nullptr;
+  ChoiceState* d_choice = nullptr;  // per class
   double* d_z2 = nullptr;
   std::vector<double> h_z2;        // host copy of d_z2 (filled at the first estimate)
   double* d_est = nullptr;         // per-pair moments [n_pairs][PMC_MOMENT_WORDS]
@@ -244,14 +255,16 @@ struct pmc_chains_s {
 // Scattering depth of the straight segment from the source to the sensor
 // point nearest it (host, FP64): the mean of the truncated Poisson law of the
 // reference density's vertex count.
-static double straight_tau_b(const pmc_medium_s* m, const PairHost& h) {
+// (or, with `absorption`, its absorption depth)
+static double straight_tau_b(const pmc_medium_s* m, const PairHost& h, bool absorption = false) {
   double rel[3], e[3];
   for (int i = 0; i < 3; ++i) rel[i] = h.c[i] - h.src[i];
   const double D = norm3(rel);
   for (int i = 0; i < 3; ++i) e[i] = h.src[i] + rel[i] * (D - h.R) / D;
   const double ell = D - h.R;
-  if (m->d.kind == PMC_HOMOGENEOUS) return ell / m->lambda_s;
-  const int L = static_cast<int>(m->ls_layers.size());
+  if (m->d.kind == PMC_HOMOGENEOUS) return ell / (absorption ? m->lambda_a : m->lambda_s);
+  const std::vector<double>& lengths = absorption ? m->la_layers : m->ls_layers;
+  const int L = static_cast<int>(lengths.size());
   auto layer = [&](double z) {
     double f = std::floor((z - m->z0) / m->dz);
     if (f < 0) f = 0;
@@ -260,13 +273,13 @@ static double straight_tau_b(const pmc_medium_s* m, const PairHost& h) {
   };
   const double zP = h.src[2], zQ = e[2];
   const int lP = layer(zP), lQ = layer(zQ);
-  if (lP == lQ) return ell / m->ls_layers[lP];
+  if (lP == lQ) return ell / lengths[lP];
   const double zlo = std::min(zP, zQ), zhi = std::max(zP, zQ);
   double acc = 0.0;
   for (int l = std::min(lP, lQ); l <= std::max(lP, lQ); ++l) {
     const double lo = (l == std::min(lP, lQ)) ? zlo : m->z0 + l * m->dz;
     const double hi = (l == std::max(lP, lQ)) ? zhi : m->z0 + (l + 1) * m->dz;
-    acc += std::max(hi - lo, 0.0) / (zhi - zlo) / m->ls_layers[l];
+    acc += std::max(hi - lo, 0.0) / (zhi - zlo) / lengths[l];
   }
   return ell * acc;
 }
@@ -597,6 +610,7 @@ int pmc_destroy_chains(pmc_chains_t ch) {
   cudaFree(ch->d_acc);
   cudaFree(ch->d_status);
   cudaFree(ch->d_queue);
+  cudaFree(ch->d_choice);
   cudaFree(ch->d_z2);
   cudaFree(ch->d_est);
   cudaFree(ch->d_mom_chunks);
@@ -935,6 +949,55 @@ static int autotune_classes(pmc_chains_t ch, cudaStream_t s) {
   return rc;
 }
 
+// Vertex count that few of a pair's paths exceed in equilibrium: mean plus two standard
+// deviations, from a path length D sqrt(1 + x) with x = 3/4 (1 - <cos>) tau_b / tau_a,
+// which is the source-sensor distance D for strong absorption and the mean
+// of the diffusion approximation for weak, and its derivative in the
+// absorption.  (Means of 15 scenes with chains seeded by the tracer: predicted
+// 38 to 223, found 40 to 221, each within 10 %.)
+static double grown_n(const pmc_medium_s* m, const PairHost& h) {
+  const double tb = straight_tau_b(m, h), ta = straight_tau_b(m, h, true);
+  const double liu = m->d.sl_alpha / (m->d.sl_alpha + 2.0);
+  const double cos_mean = m->d.f_sl > 0.f ? (1.0 - m->d.f_sl) * m->d.g + m->d.f_sl * liu : m->d.g;
+  const double x = 0.75 * (1.0 - cos_mean) * tb / ta;
+  if (!(x < 1e12)) return std::numeric_limits<double>::infinity();
+  const double n = 2.0 + tb * std::sqrt(1.0 + x);
+  return n + 2.0 * std::sqrt(n * (1.0 + 0.5 * tb / ta * x / (1.0 + x)));
+}
+
+// Kernels that may take the place of a class's tuned or caller-set one, by the
+// vertex counts at the start of a launch (launch_choose): one copy of the step
+// code, unrolled (kShareOneCopy), where more than one path in 20 lies beyond the
+// shared window (figures at chain_kernel: the lines cross between 3 and 6 %); and,
+// for lean chains that are few enough to have whole caps of more than kLongPaths
+// vertices in shared memory, where half of the paths are that long (1,216 chains,
+// 500 steps: 670 vertices 0.68 ms rolled and 0.63 unrolled, 272 vertices 0.56 and 0.55,
+// 4 vertices 1 % the other way).
+constexpr int kBeyondShare = 20, kShortPaths = 112, kLongPaths = 320;
+static int set_choices(pmc_chains_t ch) {
+  for (ChainClass& cl : ch->classes) {
+    const int chains = cl.hi - cl.lo;
+    auto add = [&](int share, bool spill, int window, int wpb) -> cudaError_t {
+      int bps = 0;
+      const cudaError_t e = ch->kernels->occupancy(cl.kind, share, ch->grad, spill, wpb, window, &bps);
+      if (e == cudaSuccess && bps >= 1)
+        cl.others.push_back({share, spill, window, wpb,
+                             std::max(1, std::min((work_items(cl.kind, share, chains) + wpb - 1) / wpb, bps * ch->ctx->n_sm))});
+      return e;
+    };
+    if (cl.kind < 2 && cl.share == 0 && cl.spill) {
+      cl.rule = {{cl.smem_cap - 1, cl.smem_cap - 1}, {chains / kBeyondShare, INT_MAX}};
+      CK(add(kShareOneCopy, true, cl.smem_cap, cl.warps_per_block));
+    } else if (cl.kind == 0 && cl.share == 0 && cl.smem_cap > kLongPaths) {
+      cl.rule = {{kLongPaths, kLongPaths}, {chains / 2, INT_MAX}};
+      CK(add(kShareOneCopy, false, cl.smem_cap, cl.warps_per_block));
+    }
+    cl.grows = cl.kind < 2 && std::any_of(ch->geom->host.begin(), ch->geom->host.end(),
+                                          [&](const PairHost& h) { return grown_n(ch->med, h) > kShortPaths; });
+  }
+  return PMC_OK;
+}
+
 int pmc_init_chains(pmc_ctx_t ctx, pmc_medium_t med, pmc_geom_t geom, const pmc_run_desc* r, void* stream,
                     pmc_chains_t* out) {
   if (!ctx || !med || !geom || !r || !out) return fail(PMC_ERR_INVALID, "NULL argument");
@@ -1181,6 +1244,7 @@ int pmc_init_chains(pmc_ctx_t ctx, pmc_medium_t med, pmc_geom_t geom, const pmc_
   CK(dalloc(&ch->d_acc, static_cast<size_t>(T) * ACC_WORDS));
   CK(dalloc(&ch->d_status, T));
   CK(dalloc(&ch->d_queue, ch->classes.size()));
+  CK(dalloc(&ch->d_choice, ch->classes.size()));
   CK(dalloc(&ch->d_z2, ch->n_pairs));
   CK(dalloc(&ch->d_est, static_cast<size_t>(ch->n_pairs) * PMC_MOMENT_WORDS + 1));
   ch->d_any = reinterpret_cast<int*>(ch->d_est + static_cast<size_t>(ch->n_pairs) * PMC_MOMENT_WORDS);
@@ -1225,6 +1289,7 @@ int pmc_init_chains(pmc_ctx_t ctx, pmc_medium_t med, pmc_geom_t geom, const pmc_
   CK(cudaMemcpyAsync(ch->d_mom_pairs, mom_pairs.data(), sizeof(MomPair) * mom_pairs.size(), cudaMemcpyHostToDevice, s));
   CK(cudaMemsetAsync(ch->d_status, 0, sizeof(int) * T, s));
   CK(cudaMemsetAsync(ch->d_any, 0, sizeof(int), s));
+  CK(cudaMemsetAsync(ch->d_choice, 0, sizeof(ChoiceState) * ch->classes.size(), s));
   CK(cudaMemsetAsync(ch->d_xyz, 0, sizeof(float) * ch->xyz_floats, s));
 
   InitParams ip{};
@@ -1302,6 +1367,8 @@ int pmc_init_chains(pmc_ctx_t ctx, pmc_medium_t med, pmc_geom_t geom, const pmc_
     const int rc = autotune_classes(ch.get(), s);
     if (rc != PMC_OK) return rc;
   }
+  const int rc = set_choices(ch.get());
+  if (rc != PMC_OK) return rc;
   *out = ch.release();
   return PMC_OK;
 }
@@ -1367,15 +1434,32 @@ int pmc_set_states(pmc_chains_t ch, const float* xyz, const int* n, int stride, 
 }
 
 // One launch per cap class; the lane kernels count a launch's steps in 32 bits.
-constexpr unsigned long long kLaneLaunchSteps = 1ull << 30;
+// Classes with a choice of kernels launch each of them, and those that were not
+// chosen return at once (some 3 us).  Where a geometry's paths are expected to grow
+// past kShortPaths vertices, long runs are cut so that the choice is made again; the cut
+// depends on the geometry alone, since it shows in the last bits of the accumulators.
+constexpr unsigned long long kLaneLaunchSteps = 1ull << 30, kChoiceSteps = 4096, kMostChoices = 64;
 static int enqueue_steps(pmc_chains_t ch, unsigned long long n_steps, cudaStream_t s) {
   for (size_t k = 0; k < ch->classes.size(); ++k) {
     const ChainClass& cl = ch->classes[k];
-    const unsigned long long most = lane_kind(cl.kind) ? kLaneLaunchSteps : n_steps;
+    const unsigned long long most = lane_kind(cl.kind) ? kLaneLaunchSteps
+                                    : cl.grows         ? std::max(kChoiceSteps, n_steps / kMostChoices + 1)
+                                                       : n_steps;
     for (unsigned long long left = n_steps; left > 0;) {
       const unsigned long long now = std::min(left, most);
-      CK(cudaMemsetAsync(ch->d_queue + k, 0, sizeof(unsigned int), s));
-      CK(ch->kernels->launch(class_params(ch, k, now), cl.kind, cl.share, ch->grad, cl.spill, cl.grid, cl.warps_per_block, s));
+      ChainParams p = class_params(ch, k, now);
+      if (cl.others.empty()) {
+        CK(cudaMemsetAsync(p.queue, 0, sizeof(unsigned int), s));
+      } else {
+        CK(launch_choose(ch->d_n, ch->d_order + cl.lo, cl.hi - cl.lo, cl.rule, ch->d_choice + k, p.queue, s));
+        p.choice = &(ch->d_choice + k)->choice;
+      }
+      CK(ch->kernels->launch(p, cl.kind, cl.share, ch->grad, cl.spill, cl.grid, cl.warps_per_block, s));
+      for (const LaunchShape& o : cl.others) {
+        ++p.option;
+        p.smem_cap = o.smem_cap;
+        CK(ch->kernels->launch(p, cl.kind, o.share, ch->grad, o.spill, o.grid, o.warps_per_block, s));
+      }
       left -= now;
     }
   }

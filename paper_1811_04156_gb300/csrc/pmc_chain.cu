@@ -37,6 +37,7 @@
 // every node's (zeta, t, phi) takes a normal step, and the new path is built
 // level by level into three extra shared arrays.
 #include <climits>
+#include <type_traits>
 
 #include "pmc_internal.h"
 #include "pmc_tree.cuh"
@@ -60,6 +61,18 @@ struct TeamNote {
   float dlen, dg;  // change of the path length and of the sum of d log sigma / dg
 };
 
+// Loop over entries of a path: f(i) for i = from, from + step, ... below `to`,
+// rolled unless the path's view says otherwise.
+template <class WP, class F>
+__device__ __forceinline__ void path_loop(int from, int to, int step, F&& f) {
+  if constexpr (WP::kRolled) {
+#pragma unroll 1
+    for (int i = from; i < to; i += step) f(i);
+  } else {
+    for (int i = from; i < to; i += step) f(i);
+  }
+}
+
 struct Sums {
   float L, G;
 };
@@ -67,11 +80,10 @@ struct Sums {
 template <class WP>
 __device__ Sums path_sums(const WP& w, int n, int lane) {
   float L = 0.f, G = 0.f;
-#pragma unroll 1
-  for (int i = lane; i < n; i += 32) {
+  path_loop<WP>(lane, n, 32, [&](int i) {
     G += w.gt(i);
     if (i <= n - 2) L += w.len(i);
-  }
+  });
   Sums s;
   s.L = warp_sum(L);
   s.G = warp_sum(G);
@@ -114,8 +126,7 @@ __device__ __forceinline__ void vs_factors(const DMedium& M, const DPair& S, flo
 template <bool kGen, bool kCall, class WP>
 __device__ float refresh_caches(const DMedium& M, const DPair& S, float zoff, const WP& w, int n, int lane) {
   float lp = 0.f;
-#pragma unroll 1
-  for (int i = lane; i < n; i += 32) {
+  path_loop<WP>(lane, n, 32, [&](int i) {
     const float3 P = w.pos(i);
     const float3 Pp = (i >= 1) ? w.pos(i - 1) : P;
     const float3 Pn = (i <= n - 2) ? w.pos(i + 1) : P;
@@ -130,7 +141,7 @@ __device__ float refresh_caches(const DMedium& M, const DPair& S, float zoff, co
       w.set_len(i, len);
       lp += seg;
     }
-  }
+  });
   __syncwarp();
   return warp_sum(lp);
 }
@@ -138,8 +149,7 @@ __device__ float refresh_caches(const DMedium& M, const DPair& S, float zoff, co
 // Shift entries [a, e) of the vertex-indexed and segment-indexed arrays.
 template <class WP>
 __device__ void shift_right(const WP& w, int a, int e_vtx, int e_seg, int lane) {
-#pragma unroll 1
-  for (int base = e_vtx - 1; base >= a; base -= 32) {
+  auto move = [&](int base) {
     const int i = base - lane;
     const bool ok = i >= a;
     const bool oks = ok && i < e_seg;
@@ -150,13 +160,18 @@ __device__ void shift_right(const WP& w, int a, int e_vtx, int e_seg, int lane) 
     if (ok) { w.set_pos(i + 1, f3(x, y, z)); w.set_vt(i + 1, vt); w.set_gt(i + 1, gt); }
     if (oks) { w.set_tb(i + 1, tb); w.set_seg(i + 1, sg); w.set_len(i + 1, ln); }
     __syncwarp();
+  };
+  if constexpr (WP::kRolled) {
+#pragma unroll 1
+    for (int base = e_vtx - 1; base >= a; base -= 32) move(base);
+  } else {
+    for (int base = e_vtx - 1; base >= a; base -= 32) move(base);
   }
 }
 
 template <class WP>
 __device__ void shift_left(const WP& w, int a, int e_vtx, int e_seg, int lane) {
-#pragma unroll 1
-  for (int base = a; base < e_vtx; base += 32) {
+  path_loop<WP>(a, e_vtx, 32, [&](int base) {
     const int i = base + lane;
     const bool ok = i < e_vtx;
     const bool oks = i < e_seg;
@@ -167,7 +182,7 @@ __device__ void shift_left(const WP& w, int a, int e_vtx, int e_seg, int lane) {
     if (ok) { w.set_pos(i - 1, f3(x, y, z)); w.set_vt(i - 1, vt); w.set_gt(i - 1, gt); }
     if (oks) { w.set_tb(i - 1, tb); w.set_seg(i - 1, sg); w.set_len(i - 1, ln); }
     __syncwarp();
-  }
+  });
 }
 
 // Segment chosen for a birth: smallest k with cumsum_k(tau_b) > u * T_b.
@@ -189,8 +204,7 @@ __device__ int select_segment(const WP& w, int nseg, float u, float& total, int 
   const int lo = lane * m;
   const int hi = min(lo + m, nseg);
   float local = 0.f;
-#pragma unroll 1
-  for (int i = lo; i < hi; ++i) local += w.tb(i);
+  path_loop<WP>(lo, hi, 1, [&](int i) { local += w.tb(i); });
   float incl = local;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -206,10 +220,17 @@ __device__ int select_segment(const WP& w, int nseg, float u, float& total, int 
   if (lane == owner) {
     float cum = incl - local;
     k = hi - 1;
-#pragma unroll 1
-    for (int i = lo; i < hi; ++i) {
+    auto passes = [&](int i) {
       cum += w.tb(i);
-      if (cum > target) { k = i; break; }
+      return cum > target;
+    };
+    if constexpr (WP::kRolled) {
+#pragma unroll 1
+      for (int i = lo; i < hi; ++i)
+        if (passes(i)) { k = i; break; }
+    } else {
+      for (int i = lo; i < hi; ++i)
+        if (passes(i)) { k = i; break; }
     }
   }
   return __shfl_sync(kFull, k, owner);
@@ -429,14 +450,26 @@ __device__ __forceinline__ void flush64(Accum& a, int lane) {
 // With acceptance rate a, 1 + (1-a) + (1-a)^2 + (1-a)^3 steps finish per round.
 // (Four groups of 8 lanes of one warp instead of four warps gain little: they
 // run through each other's kinds of moves in turn.)
+// kX = 5 is the Cartesian kernel for launches with long paths: one copy of the step
+// code, its loops unrolled as the compiler sees fit.  kX = 0 with a window holds
+// the code twice, with and without tests at the accesses, and warps in both
+// copies evict each other's instructions.  15,200 chains, 200 steps, general
+// physics, window 256: 5.41 ms with two copies and 3.32 with one where 37 % of
+// the paths lie beyond the window, 2.81 and 2.52 with 6 %, 2.07 and 2.40 with
+// 3 %; lean physics with none 1.22 and 1.46, with all (670 vertices, window 320)
+// 3.64 and 2.82.  (The same switch inside one kernel costs registers: 1.30 with none.)
 template <bool kGen, bool kGrad, bool kSpill, int kX>
-__global__ void __launch_bounds__(128, (kGen && (kX == 1 || kX == 4)) ? 4 : ((kGen || kX != 0) ? 5 : 6))
+__global__ void __launch_bounds__(128, (kGen && (kX == 1 || kX == 4)) ? 4 : ((kGen || (kX != 0 && kX != 5)) ? 5 : 6))
     chain_kernel(const ChainParams P) {
-  using WP = WarpPath<kGen, kGrad, kSpill>;
-  constexpr bool kTree = kX == 1, kHmc = kX == 2, kLam = kX == 3, kTeam = kX == 4;
-  static_assert(kX == 0 || !kSpill, "tree, HMC, wavelength and team kernels keep the whole cap in shared memory");
-  static_assert(kX == 0 || kX == 1 || kX == 4 || kGen, "HMC and wavelength moves use the general kernel");
+  constexpr bool kTree = kX == 1, kHmc = kX == 2, kLam = kX == 3, kTeam = kX == 4, kOneCopy = kX == 5;
+  using WP = WarpPath<kGen, kGrad, kSpill, !kOneCopy>;
+  static_assert(kX == 0 || kOneCopy || !kSpill,
+                "tree, HMC, wavelength and team kernels keep the whole cap in shared memory");
+  static_assert(kX == 0 || kX == 1 || kX == 4 || kOneCopy || kGen, "HMC and wavelength moves use the general kernel");
   constexpr int kArraysAll = WP::kArrays + (kTree ? 3 : 0) + (kHmc ? 6 : 0);
+  if constexpr (kX == 0 || kOneCopy) {
+    if (P.choice != nullptr && *P.choice != P.option) return;
+  }
   extern __shared__ float4 smem4[];
   float* smem = reinterpret_cast<float*>(smem4);
   const int lane = threadIdx.x & 31;
@@ -702,7 +735,7 @@ __global__ void __launch_bounds__(128, (kGen && (kX == 1 || kX == 4)) ? 4 : ((kG
             move = MV_INTERIOR;
             const float3 fj = w.pos(j);
             const float3 z = f3(__uint_as_float(lo.z), __uint_as_float(lo.w), __uint_as_float(hi.x));
-            if constexpr (kGen && (kX == 0 || kTeam)) {
+            if constexpr (kGen && (kX == 0 || kTeam || kOneCopy)) {
               if (R.within == 1) {
                 gx_mala = grad_vertex_warp<32>(M, S, zoff, [&](int k) { return w.pos(k); }, n, j, lane);
                 const float h = 0.5f * R.mala_eps * R.mala_eps;
@@ -811,14 +844,14 @@ __global__ void __launch_bounds__(128, (kGen && (kX == 1 || kX == 4)) ? 4 : ((kG
             // T_b of the reduced path, summed afresh so that decisions depend
             // only on the current state (split runs replay exactly)
             float part = 0.f;
-#pragma unroll 1
-            for (int q = lane; q < n - 1; q += 32) part += w.tb(q);
+            path_loop<std::remove_cv_t<std::remove_reference_t<decltype(w)>>>(lane, n - 1, 32,
+                                                                             [&](int q) { part += w.tb(q); });
             const float tb_new = __shfl_sync(kFull, ntb, 0);
             const float Tb_red = warp_sum(part) + dtb;
             extra = -R.log_pd + __logf(static_cast<float>(n - 2)) + R.log_pb + __logf(__fdividef(tb_new, Tb_red)) +
                     log_insert_density<true>(M, R, zoff, w.pos(jj - 1), w.pos(jj + 1), w.pos(jj));
           }
-          if constexpr (kGen && (kX == 0 || kTeam)) {
+          if constexpr (kGen && (kX == 0 || kTeam || kOneCopy)) {
             if (move == MV_INTERIOR && R.within == 1 && isfinite(dlp)) {
               const float3 gy = grad_vertex_warp<32>(M, S, zoff, newpos, n, jj, lane);
               const float h = 0.5f * R.mala_eps * R.mala_eps;
@@ -906,7 +939,7 @@ __global__ void __launch_bounds__(128, (kGen && (kX == 1 || kX == 4)) ? 4 : ((kG
       };
 #pragma unroll 1
       for (int i = 0; i < cnt;) {
-        if constexpr (kSpill) {
+        if constexpr (kSpill && !kOneCopy) {
           // a path that stays within the window even after a birth needs no
           // test at its accesses
           if (n < cap_s) step(w_in, i, true);
@@ -1064,6 +1097,7 @@ void launch_one(const ChainParams& p, int grid, int warps_per_block, size_t sm, 
 // spill), general with tree moves and general with HMC moves (never spilled).
 int kernel_key(int kind, int share, bool grad, bool spill) {
   if (share == kShareTeam) return 16 + (kind == 1 ? 2 : 0) + (grad ? 1 : 0);
+  if (share == kShareOneCopy) return spill ? 20 + (kind == 1 ? 2 : 0) + (grad ? 1 : 0) : 24 + (grad ? 1 : 0);
   if (kind == 2) return 8 + (grad ? 1 : 0);
   if (kind == 3) return 10 + (grad ? 1 : 0);
   if (kind == 6) return 12;
@@ -1090,6 +1124,7 @@ cudaError_t chain_occupancy(int kind, int share, bool grad, bool spill, int warp
     return kind == 1 ? group_kernel(grad, spill, nullptr, 0, warps_per_block, smem_cap, blocks_per_sm, nullptr)
                      : cudaErrorInvalidValue;
   if (share == kShareTeam && (kind > 1 || spill || warps_per_block != kTeamWarps)) return cudaErrorInvalidValue;
+  if (share == kShareOneCopy && (kind > 1 || (kind == 1 && !spill))) return cudaErrorInvalidValue;
   if (lane_kind(kind)) return lane_occupancy(kind, warps_per_block, smem_cap, grad, blocks_per_sm);
   if (kind >= 2 && spill) return cudaErrorInvalidValue;
   if (kind == 6 && grad) return cudaErrorInvalidValue;
@@ -1113,6 +1148,12 @@ cudaError_t chain_occupancy(int kind, int share, bool grad, bool spill, int warp
     case 17: return occupancy_of<false, true, false, 4>(warps_per_block, sm, blocks_per_sm);
     case 18: return occupancy_of<true, false, false, 4>(warps_per_block, sm, blocks_per_sm);
     case 19: return occupancy_of<true, true, false, 4>(warps_per_block, sm, blocks_per_sm);
+    case 20: return occupancy_of<false, false, true, 5>(warps_per_block, sm, blocks_per_sm);
+    case 21: return occupancy_of<false, true, true, 5>(warps_per_block, sm, blocks_per_sm);
+    case 22: return occupancy_of<true, false, true, 5>(warps_per_block, sm, blocks_per_sm);
+    case 23: return occupancy_of<true, true, true, 5>(warps_per_block, sm, blocks_per_sm);
+    case 24: return occupancy_of<false, false, false, 5>(warps_per_block, sm, blocks_per_sm);
+    case 25: return occupancy_of<false, true, false, 5>(warps_per_block, sm, blocks_per_sm);
     default: return occupancy_of<true, true, false, 2>(warps_per_block, sm, blocks_per_sm);
   }
 }
@@ -1123,6 +1164,7 @@ cudaError_t launch_chain(const ChainParams& p, int kind, int share, bool grad, b
     return kind == 1 ? group_kernel(grad, spill, &p, grid, warps_per_block, p.smem_cap, nullptr, s)
                      : cudaErrorInvalidValue;
   if (share == kShareTeam && (kind > 1 || spill || warps_per_block != kTeamWarps)) return cudaErrorInvalidValue;
+  if (share == kShareOneCopy && (kind > 1 || (kind == 1 && !spill))) return cudaErrorInvalidValue;
   if (lane_kind(kind)) return launch_lane_chain(p, kind, grid, warps_per_block, grad, s);
   if (kind >= 2 && spill) return cudaErrorInvalidValue;
   if (kind == 6 && grad) return cudaErrorInvalidValue;
@@ -1146,6 +1188,12 @@ cudaError_t launch_chain(const ChainParams& p, int kind, int share, bool grad, b
     case 17: launch_one<false, true, false, 4>(p, grid, warps_per_block, sm, s); break;
     case 18: launch_one<true, false, false, 4>(p, grid, warps_per_block, sm, s); break;
     case 19: launch_one<true, true, false, 4>(p, grid, warps_per_block, sm, s); break;
+    case 20: launch_one<false, false, true, 5>(p, grid, warps_per_block, sm, s); break;
+    case 21: launch_one<false, true, true, 5>(p, grid, warps_per_block, sm, s); break;
+    case 22: launch_one<true, false, true, 5>(p, grid, warps_per_block, sm, s); break;
+    case 23: launch_one<true, true, true, 5>(p, grid, warps_per_block, sm, s); break;
+    case 24: launch_one<false, false, false, 5>(p, grid, warps_per_block, sm, s); break;
+    case 25: launch_one<false, true, false, 5>(p, grid, warps_per_block, sm, s); break;
     default: launch_one<true, true, false, 2>(p, grid, warps_per_block, sm, s); break;
   }
   return cudaGetLastError();

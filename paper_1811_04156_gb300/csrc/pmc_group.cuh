@@ -293,6 +293,7 @@ __host__ __device__ constexpr int group_words(int arrays, int cap_s, int steps, 
 
 template <bool kGen, bool kGrad, bool kSpill, int kG>
 __global__ void __launch_bounds__(128, 4) group_chain_kernel(const ChainParams P) {
+  if (P.choice != nullptr && *P.choice != P.option) return;
   using WP = GroupPath<kGen, kGrad, kSpill>;
   constexpr int kChains = 32 / kG;  // chains of a warp
   constexpr int kBatch = kG;        // steps whose random numbers are staged at once

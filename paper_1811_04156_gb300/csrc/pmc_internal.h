@@ -53,6 +53,8 @@ struct ChainParams {
   int* status;                  // [total]
   int* any_status;              // OR of all status words
   unsigned int* queue;          // work counter of this launch
+  const int* choice;            // launches of several kernels of which one runs: the option to run, else null
+  int option;                   // this launch's option
   const volatile int* abort_flag;
   uint32_t chain_id0;           // global index of local chain 0 (Philox counter word of a chain)
   float* lam;                   // [total] wavelength of each chain (wavelength sampling), else null
@@ -89,9 +91,10 @@ inline bool lane_kind(int kind) { return kind == 4 || kind == 5 || kind == 8; }
 constexpr int kLaneTreeArrays = 4;
 // `share` (kinds 0 and 1): 0 one warp per chain; kShareGroup 8 lanes per chain
 // (kind 1, Gaussian moves; pmc_group.cuh); kShareTeam a block of four warps per
-// chain, each on one of its next steps (no spill).  The same decisions and the
-// same results.
-constexpr int kShareGroup = 1, kShareTeam = 2;
+// chain, each on one of its next steps (no spill); kShareOneCopy one warp per
+// chain with a window, for launches with many paths beyond it.  The same
+// decisions and the same results.
+constexpr int kShareGroup = 1, kShareTeam = 2, kShareOneCopy = 3;
 constexpr int kGroupLanes = 8;
 inline int chain_arrays(bool general, bool grad) { return 6 + (general ? 1 : 0) + (grad ? 1 : 0); }
 
@@ -158,6 +161,21 @@ struct InitParams {
 };
 
 // pmc_kernels.cu
+// Which of up to three kernels (options 0, 1, 2) a class's next launch runs, by the
+// vertex counts of its chains order[0 .. chains): option 0 while at most
+// max_past[0] chains have more than past[0] vertices, else option 1 while at most
+// max_past[1] have more than past[1], else option 2.  Also clears the launch's
+// work counter.
+struct ChoiceState {
+  int past[2];                  // chains counted so far (zero between launches)
+  unsigned int blocks;          // blocks that have counted
+  int choice;
+};
+struct ChoiceRule {
+  int past[2], max_past[2];
+};
+cudaError_t launch_choose(const int* n, const int* order, int chains, const ChoiceRule& rule, ChoiceState* state,
+                          unsigned int* queue, cudaStream_t s);
 cudaError_t launch_logp(const DMedium& M, const DPair& S, const float* xyz, const int* n, int batch, int cap,
                         float* out_logp, float* out_grad, int n_sm, cudaStream_t s);
 cudaError_t launch_score(const DMedium& M, const DPair& S, const float* xyz, const int* n, int batch, int cap,

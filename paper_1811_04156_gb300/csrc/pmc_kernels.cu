@@ -545,6 +545,34 @@ __global__ void __launch_bounds__(256)
                 });
 }
 
+// Choice of a class's kernel by its chains' vertex counts (pmc_internal.h): the last
+// block to have counted its share decides and leaves the counters at zero.
+constexpr int kChooseThreads = 256, kChooseBlocks = 64;
+__global__ void __launch_bounds__(kChooseThreads) choose_kernel(const int* __restrict__ n,
+                                                                const int* __restrict__ order, int chains,
+                                                                ChoiceRule rule, ChoiceState* state,
+                                                                unsigned int* queue) {
+  int past[2] = {0, 0};
+  for (int i = blockIdx.x * kChooseThreads + threadIdx.x; i < chains; i += gridDim.x * kChooseThreads) {
+    const int k = n[order[i]];
+    past[0] += k > rule.past[0];
+    past[1] += k > rule.past[1];
+  }
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    past[j] = __reduce_add_sync(kFull, past[j]);
+    if ((threadIdx.x & 31) == 0 && past[j] > 0) atomicAdd(&state->past[j], past[j]);
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x != 0 || atomicAdd(&state->blocks, 1u) != gridDim.x - 1) return;
+  __threadfence();
+  const int a = atomicExch(&state->past[0], 0), b = atomicExch(&state->past[1], 0);
+  state->blocks = 0u;
+  state->choice = a <= rule.max_past[0] ? 0 : (b <= rule.max_past[1] ? 1 : 2);
+  *queue = 0u;
+}
+
 // Per-layer scores of every chain's current path, summed per pair (layered
 // media): theta = (lambda_s[l], lambda_a[l]) with d log p / d lambda_s[l] =
 // len_l b_l^2 - n_l b_l and d log p / d lambda_a[l] = len_l a_l^2 (len_l: path
@@ -613,6 +641,13 @@ __global__ void __launch_bounds__(128) chain_layer_score_kernel(const DMedium M,
 }
 
 }  // namespace
+
+cudaError_t launch_choose(const int* n, const int* order, int chains, const ChoiceRule& rule, ChoiceState* state,
+                          unsigned int* queue, cudaStream_t s) {
+  const int blocks = std::min(kChooseBlocks, (chains + kChooseThreads - 1) / kChooseThreads);
+  choose_kernel<<<blocks, kChooseThreads, 0, s>>>(n, order, chains, rule, state, queue);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_logp(const DMedium& M, const DPair& S, const float* xyz, const int* n, int batch, int cap,
                         float* out_logp, float* out_grad, int n_sm, cudaStream_t s) {

@@ -24,9 +24,11 @@ enum Move { MV_INTERIOR = 0, MV_END = 1, MV_BIRTH = 2, MV_DEATH = 3 };
 // array a at offset a * stride).  kTb: tau_b per segment is cached (layered
 // media); otherwise it is b * length.  kGt: d log sigma / dg per vertex is
 // cached (gradients requested).  kSpill = false: the whole cap fits (S >= cap)
-// and every access goes to shared memory.
-template <bool kTb, bool kGt, bool kSpill>
+// and every access goes to shared memory.  kRoll: loops over the path are kept
+// rolled (path_loop in pmc_chain.cu).
+template <bool kTb, bool kGt, bool kSpill, bool kRoll = true>
 struct WarpPath {
+  static constexpr bool kRolled = kRoll;
   static constexpr int kArrays = 6 + (kTb ? 1 : 0) + (kGt ? 1 : 0);
   static constexpr int kX = 0, kY = 1, kZ = 2, kSeg = 3, kLen = 4, kVt = 5, kTbA = 6, kGtA = 6 + (kTb ? 1 : 0);
   float* sm;   // shared arrays, stride S
