@@ -764,8 +764,9 @@ static bool fused_births(pmc_chains_t ch, const ChainClass& cl) {
 // whose paths are expected to stay within the groups' window (the straight
 // line's vertex count); 30,720 chains of 44 vertices in 100 layers, 500 steps:
 // 10.3 ms with one warp per chain (window 256), 6.9 ms in groups (window 128;
-// 8.4 with 96, 9.3 with 192; 6.2 flushing subnormals).  The lean kernel's longer paths spill there
-// (40 against 30 ms).  Teams: offered to the autotuner up to four chains per SM
+// 8.4 with 96, 9.3 with 192; 6.2 flushing subnormals).  Paths grow longer than the
+// straight line's, so each launch may take a warp per chain instead (set_choices).
+// The lean kernel's longer paths spill there (40 against 30 ms).  Teams: offered to the autotuner up to four chains per SM
 // (one warp per scheduler); 1,000 plain steps of 64 chains 0.94 ms with one warp
 // per chain, 0.75 with teams, of 608 chains 0.96 and 0.93, of 912 1.01 and 1.57
 // (100 layers: 1.39 and 1.16, 1.41 and 1.45, 1.49 and 2.55).
@@ -972,8 +973,18 @@ static double grown_n(const pmc_medium_s* m, const PairHost& h) {
 // for lean chains that are few enough to have whole caps of more than kLongPaths
 // vertices in shared memory, where half of the paths are that long (1,216 chains,
 // 500 steps: 670 vertices 0.68 ms rolled and 0.63 unrolled, 272 vertices 0.56 and 0.55,
-// 4 vertices 1 % the other way).
+// 4 vertices 1 % the other way).  Groups of 8 lanes give way to a warp per chain
+// where more than one path in 64 has outgrown their window, or with less than 64
+// chains per SM, where a launch waits for its slowest warp, one in 1,024.  200 steps
+// of 100 and of 24 chains per SM, groups and the warp layout:
+//   paths beyond 128      0.4 %        1.3 %        5 %          10 %         62 %
+//   100 per SM, groups    1.35 ms      1.51         2.2          2.65         8.5
+//               warps     1.52         1.62         1.6          1.64         3.2
+//    24 per SM, groups    0.71         0.82         0.99         1.13         5.4
+//               warps     0.52         0.54         0.53         0.56         1.2
+// (none beyond: 1.20 and 1.58; 0.52 and 0.53).
 constexpr int kBeyondShare = 20, kShortPaths = 112, kLongPaths = 320;
+constexpr int kManyGroups = 64, kLongShareMany = 64, kLongShare = 1024;
 static int set_choices(pmc_chains_t ch) {
   for (ChainClass& cl : ch->classes) {
     const int chains = cl.hi - cl.lo;
@@ -991,6 +1002,12 @@ static int set_choices(pmc_chains_t ch) {
     } else if (cl.kind == 0 && cl.share == 0 && cl.smem_cap > kLongPaths) {
       cl.rule = {{kLongPaths, kLongPaths}, {chains / 2, INT_MAX}};
       CK(add(kShareOneCopy, false, cl.smem_cap, cl.warps_per_block));
+    } else if (cl.share == kShareGroup && cl.spill) {
+      const int full = (cl.max_cap + 31) / 32 * 32, window = warp_window(ch, full, chains);
+      const int few = chains >= kManyGroups * ch->ctx->n_sm ? kLongShareMany : kLongShare;
+      cl.rule = {{kGroupWindow - 2, window - 1}, {chains / few, window < full ? chains / kBeyondShare : INT_MAX}};
+      CK(add(0, window < full, window, 4));
+      if (window < full) CK(add(kShareOneCopy, true, window, 4));
     }
     cl.grows = cl.kind < 2 && std::any_of(ch->geom->host.begin(), ch->geom->host.end(),
                                           [&](const PairHost& h) { return grown_n(ch->med, h) > kShortPaths; });

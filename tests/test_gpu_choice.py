@@ -81,3 +81,25 @@ def test_long_runs_are_cut_without_a_trace():
     assert np.allclose(whole[3], parts[3], rtol=1e-5) and whole[1].max() > 64
     (other,) = _run(sc, (9000,), warps_per_block=4, smem_window=96)
     _same([whole], [other])
+
+
+@pytest.mark.parametrize("cap,init_k", [(200, 118), (700, 20), (700, 118), (700, 200), (700, 400)])
+def test_groups_give_way_to_warps(cap, init_k):
+    """Enough general chains for groups of 8 lanes: paths inside the groups' window of 128,
+    paths that grow across it within a launch, and paths that start beyond it or
+    beyond the warp layout's window, against the warp layout set by the caller."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    sc = _scene("general", 21 * n_sm + 3, cap, init_k)
+    sc.run.init_jitter = 2e-4
+    if init_k == 118:  # (a dense medium: 101 scatterings on the straight line, paths grow)
+        sc.medium = S.Medium(lambda_s=0.0125, lambda_a=100.0, g=0.2)
+        sc.run.sigma = 0.005
+    steps = (733, 35, 300)
+    a = _run(sc, steps)
+    _same(a, _run(sc, steps, warps_per_block=2))
+    assert (a[-1][3][:, 0] > 0).mean() > 0.9
+    if init_k == 118:
+        assert a[0][1].max() > 128
