@@ -49,7 +49,8 @@ def _sources():
 
 
 def _deps():
-    return _sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) + \
+    """What the library is made from, this file with its flags included."""
+    return [os.path.abspath(__file__)] + _sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) + \
         glob.glob(os.path.join(INCLUDE, "*.h"))
 
 
@@ -61,7 +62,8 @@ def up_to_date() -> bool:
 
 
 def _build_probe(nvcc: str) -> None:
-    if os.path.exists(PROBE_LIB) and os.path.getmtime(PROBE_LIB) >= os.path.getmtime(PROBE_SRC):
+    if os.path.exists(PROBE_LIB) and all(os.path.getmtime(PROBE_LIB) >= os.path.getmtime(p)
+                                         for p in (PROBE_SRC, os.path.abspath(__file__))):
         return
     tmp = PROBE_LIB + f".tmp{os.getpid()}"
     r = subprocess.run([nvcc, "-shared", "-o", tmp, PROBE_SRC] + NVCC_FLAGS, capture_output=True, text=True)
