@@ -737,7 +737,7 @@ __global__ void __launch_bounds__(128, (kGen && (kX == 1 || kX == 4)) ? 4 : ((kG
             const float3 z = f3(__uint_as_float(lo.z), __uint_as_float(lo.w), __uint_as_float(hi.x));
             if constexpr (kGen && (kX == 0 || kTeam || kOneCopy)) {
               if (R.within == 1) {
-                gx_mala = grad_vertex_warp<32>(M, S, zoff, [&](int k) { return w.pos(k); }, n, j, lane);
+                gx_mala = grad_vertex_warp(M, S, zoff, [&](int k) { return w.pos(k); }, n, j, lane);
                 const float h = 0.5f * R.mala_eps * R.mala_eps;
                 fnew = fj + h * gx_mala + R.mala_eps * z;
               } else {
@@ -853,7 +853,7 @@ __global__ void __launch_bounds__(128, (kGen && (kX == 1 || kX == 4)) ? 4 : ((kG
           }
           if constexpr (kGen && (kX == 0 || kTeam || kOneCopy)) {
             if (move == MV_INTERIOR && R.within == 1 && isfinite(dlp)) {
-              const float3 gy = grad_vertex_warp<32>(M, S, zoff, newpos, n, jj, lane);
+              const float3 gy = grad_vertex_warp(M, S, zoff, newpos, n, jj, lane);
               const float h = 0.5f * R.mala_eps * R.mala_eps;
               const float3 fj = w.pos(jj);
               const float3 dfw = fnew - fj - h * gx_mala;

@@ -7,18 +7,17 @@ namespace PMC_VARIANT {
 
 size_t group_smem_bytes(bool grad, int smem_cap, int warps_per_block) {
   return static_cast<size_t>(warps_per_block) * (32 / kGroupLanes) *
-         group_words(chain_arrays(true, grad), smem_cap, kGroupLanes, kGroupLanes) * sizeof(float);
+         group_words(chain_arrays(true, grad), smem_cap) * sizeof(float);
 }
 
 cudaError_t group_kernel(bool grad, bool spill, const ChainParams* p, int grid, int warps_per_block, int smem_cap,
                          int* blocks_per_sm, cudaStream_t s) {
   const size_t smem = group_smem_bytes(grad, smem_cap, warps_per_block);
-  constexpr int kG = kGroupLanes;
   if (spill)
-    return grad ? group_call<true, true, true, kG>(p, grid, warps_per_block, smem, blocks_per_sm, s)
-                : group_call<true, false, true, kG>(p, grid, warps_per_block, smem, blocks_per_sm, s);
-  return grad ? group_call<true, true, false, kG>(p, grid, warps_per_block, smem, blocks_per_sm, s)
-              : group_call<true, false, false, kG>(p, grid, warps_per_block, smem, blocks_per_sm, s);
+    return grad ? group_call<true, true>(p, grid, warps_per_block, smem, blocks_per_sm, s)
+                : group_call<false, true>(p, grid, warps_per_block, smem, blocks_per_sm, s);
+  return grad ? group_call<true, false>(p, grid, warps_per_block, smem, blocks_per_sm, s)
+              : group_call<false, false>(p, grid, warps_per_block, smem, blocks_per_sm, s);
 }
 
 }  // namespace PMC_VARIANT

@@ -1,7 +1,7 @@
-// RJMCMC chain kernel with a group of kG lanes of a warp per chain (Collin,
+// RJMCMC chain kernel with a group of kG = 8 lanes of a warp per chain (Collin,
 // arXiv:1811.04156: section "Numerical path integration", Eq. acceptFact;
-// appendix "Jump proposal" and "Dimension matching transformation"), for
-// Gaussian vertex moves.  The same Markov chains as the
+// appendix "Jump proposal" and "Dimension matching transformation"), for the general
+// physics with Gaussian vertex moves.  The same Markov chains as the
 // warp-per-chain kernel in pmc_chain.cu, decision for decision: the same
 // Philox counters, the same factors, and every sum over a path (T_b, the choice
 // of a birth's segment, the path length) taken in the order in which 32 lanes
@@ -29,19 +29,17 @@ namespace {
 
 // View of one chain's path: entries [0, S) live in the warp's shared memory,
 // [vertex] float4 (position and vertex factor), then [segment] float2 (factor
-// and length), then the optional arrays; entries [S, cap) in the chain's global
-// block, array a at offset a * cap.  kTb: tau_b per segment is cached (layered
-// media); otherwise it is b * length.  kGt: d log sigma / dg per vertex is
+// and length), then tau_b per segment and the optional array; entries [S, cap) in
+// the chain's global block, array a at offset a * cap.  kGt: d log sigma / dg per vertex is
 // cached (gradients requested).  kSpill = false: the whole cap fits (S >= cap)
 // and every access goes to shared memory.
-template <bool kTb, bool kGt, bool kSpill>
+template <bool kGt, bool kSpill>
 struct GroupPath {
-  static constexpr int kArrays = 6 + (kTb ? 1 : 0) + (kGt ? 1 : 0);
-  static constexpr int kX = 0, kY = 1, kZ = 2, kSeg = 3, kLen = 4, kVt = 5, kTbA = 6, kGtA = 6 + (kTb ? 1 : 0);
+  static constexpr int kArrays = 7 + (kGt ? 1 : 0);
+  static constexpr int kX = 0, kY = 1, kZ = 2, kSeg = 3, kLen = 4, kVt = 5, kTbA = 6, kGtA = 7;
   float* sm;   // shared block
   float* gm;   // global block of the chain, stride cap
   int S, cap;
-  float b;
   __device__ __forceinline__ float4* va(int i) const { return reinterpret_cast<float4*>(sm) + i; }
   __device__ __forceinline__ float2* vb(int i) const { return reinterpret_cast<float2*>(sm + 4 * S) + i; }
   template <int a>
@@ -102,21 +100,16 @@ struct GroupPath {
   __device__ __forceinline__ float len(int i) const { return ld<kLen>(i); }
   __device__ __forceinline__ float vt(int i) const { return ld<kVt>(i); }
   __device__ __forceinline__ void set_vt(int i, float v) const { st<kVt>(i, v); }
-  __device__ __forceinline__ float tb(int i) const {
-    if constexpr (kTb) return ld<kTbA>(i);
-    else return b * ld<kLen>(i);
-  }
+  __device__ __forceinline__ float tb(int i) const { return ld<kTbA>(i); }
   __device__ __forceinline__ float gt(int i) const {
     if constexpr (kGt) return ld<kGtA>(i);
     else return 0.f;
   }
-  __device__ __forceinline__ void set_tb(int i, float v) const {
-    if constexpr (kTb) st<kTbA>(i, v);
-  }
+  __device__ __forceinline__ void set_tb(int i, float v) const { st<kTbA>(i, v); }
   __device__ __forceinline__ void set_gt(int i, float v) const {
     if constexpr (kGt) st<kGtA>(i, v);
   }
-  // entry i of the arrays that move with a birth or a death (tau_b cached only)
+  // entry i of the arrays that move with a birth or a death
   struct Entry {
     float4 v;
     float2 s;
@@ -130,7 +123,7 @@ struct GroupPath {
     e.tb = 0.f;
     if (segment_too) {
       e.s = segment(i);
-      if constexpr (kTb) e.tb = tb(i);
+      e.tb = tb(i);
     }
     return e;
   }
@@ -144,14 +137,14 @@ struct GroupPath {
   }
 };
 
-template <int kG>
+constexpr int kG = kGroupLanes;
+
 __device__ __forceinline__ float group_get(float v, int from) {
   return __shfl_sync(kFull, v, from, kG);
 }
 
 // Sum over the 32 virtual lanes of a group (virtual lane gl + kG * j holds
 // part[j]) in the order of a 32-lane butterfly.
-template <int kG>
 __device__ __forceinline__ float group_sum(float (&part)[32 / kG]) {
 #pragma unroll
   for (int h = 32 / kG / 2; h > 0; h >>= 1)
@@ -164,7 +157,7 @@ __device__ __forceinline__ float group_sum(float (&part)[32 / kG]) {
 }
 
 // Sum of f(i) over i < m, the terms spread over 32 virtual lanes by i mod 32.
-template <int kG, class F>
+template <class F>
 __device__ __forceinline__ float group_sum_of(int m, int gl, F&& f) {
   float part[32 / kG];
 #pragma unroll
@@ -177,13 +170,13 @@ __device__ __forceinline__ float group_sum_of(int m, int gl, F&& f) {
       if (i < m) part[j] += f(i);
     }
   }
-  return group_sum<kG>(part);
+  return group_sum(part);
 }
 
 // Segment chosen for a birth: smallest k with cumsum_k(tau_b) > u * T_b, the
 // cumulative sums as 32 lanes form them: each virtual lane v (v = gl * kV + j)
 // adds up m consecutive segments, then an inclusive scan over the lanes.
-template <int kG, class WP>
+template <class WP>
 __device__ __forceinline__ int group_select(const WP& w, int nseg, float u, float& total, int gl) {
   constexpr int kV = 32 / kG;
   const int m = (nseg + 31) >> 5;
@@ -208,7 +201,7 @@ __device__ __forceinline__ int group_select(const WP& w, int nseg, float u, floa
     for (int j = 0; j < kV; ++j)
       if (gl * kV + j >= o) incl[j] += y[j];
   }
-  total = group_get<kG>(incl[kV - 1], kG - 1);
+  total = group_get(incl[kV - 1], kG - 1);
   const float target = u * total;
   // first virtual lane past the target, else the last one that holds a segment
   int first = kV, last = -1;
@@ -219,7 +212,7 @@ __device__ __forceinline__ int group_select(const WP& w, int nseg, float u, floa
     if (has && last < 0) last = j;
   }
   const int shift = (threadIdx.x & 31) - gl;
-  constexpr unsigned kMask = kG == 32 ? 0xffffffffu : ((1u << (kG & 31)) - 1u);
+  constexpr unsigned kMask = (1u << kG) - 1u;
   const unsigned over = (__ballot_sync(kFull, first < kV) >> shift) & kMask;
   const unsigned has = (__ballot_sync(kFull, last >= 0) >> shift) & kMask;
   const int owner = over ? (__ffs(over) - 1) : (31 - __clz(has));
@@ -286,32 +279,31 @@ __device__ __forceinline__ void group_flush(GroupAcc& a, double* acc, bool write
 
 // Words of shared memory per chain: its arrays, the staged random numbers, the
 // pair constants, and a remainder that sets neighbouring chains kG banks apart.
-__host__ __device__ constexpr int group_words(int arrays, int cap_s, int steps, int lanes) {
-  const int w = arrays * cap_s + steps * kRngWords + kPairWords;
-  return w + ((lanes & 31) - w % 32 + 32) % 32;
+__host__ __device__ constexpr int group_words(int arrays, int cap_s) {
+  const int w = arrays * cap_s + kG * kRngWords + kPairWords;
+  return w + (kG - w % 32 + 32) % 32;
 }
 
-template <bool kGen, bool kGrad, bool kSpill, int kG>
+template <bool kGrad, bool kSpill>
 __global__ void __launch_bounds__(128, 4) group_chain_kernel(const ChainParams P) {
   if (P.choice != nullptr && *P.choice != P.option) return;
-  using WP = GroupPath<kGen, kGrad, kSpill>;
+  using WP = GroupPath<kGrad, kSpill>;
   constexpr int kChains = 32 / kG;  // chains of a warp
   constexpr int kBatch = kG;        // steps whose random numbers are staged at once
   extern __shared__ float4 group_smem4[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int gl = lane % kG, gi = lane / kG;
   const int cap_s = P.smem_cap;
-  const int words = group_words(WP::kArrays, cap_s, kBatch, kG);
+  const int words = group_words(WP::kArrays, cap_s);
   WP w;
   w.sm = reinterpret_cast<float*>(group_smem4) + static_cast<size_t>(wib * kChains + gi) * words;
   w.S = cap_s;
-  w.b = P.M.b;
   uint4* rng = reinterpret_cast<uint4*>(w.sm + WP::kArrays * cap_s);  // [kBatch][2]
   DPair* spair = reinterpret_cast<DPair*>(rng + 2 * kBatch);
   const DMedium& M = P.M;
   const DRun& R = P.R;
   const uint32_t key0 = static_cast<uint32_t>(R.seed), key1 = static_cast<uint32_t>(R.seed >> 32);
-  const unsigned gmask = ((1u << (kG & 31)) - 1u) << (gi * kG);  // this chain's lanes
+  const unsigned gmask = ((1u << kG) - 1u) << (gi * kG);  // this chain's lanes
 
   for (;;) {
     int item = 0;
@@ -350,7 +342,7 @@ __global__ void __launch_bounds__(128, 4) group_chain_kernel(const ChainParams P
     float* gz = gy + cap;
     w.gm = gx;
     w.cap = cap;
-    const GroupPath<kGen, kGrad, false> w_in{w.sm, w.gm, w.S, w.cap, w.b};  // the same path, all of it in the window
+    const GroupPath<kGrad, false> w_in{w.sm, w.gm, w.S, w.cap};  // the same path, all of it in the window
 #pragma unroll 1
     for (int i = gl; i < min(n, cap_s); i += kG) {
       *w.va(i) = make_float4(gx[i], gy[i], gz[i], 0.f);
@@ -364,7 +356,7 @@ __global__ void __launch_bounds__(128, 4) group_chain_kernel(const ChainParams P
       const float3 Pp = (i >= 1) ? w.pos(i - 1) : Pc;
       const float3 Pn = (i <= n - 2) ? w.pos(i + 1) : Pc;
       float vt, gt, seg, tb, len;
-      vertex_and_segment<kGen>(M, S, zoff, Pp, Pc, Pn, i, n, vt, gt, seg, tb, len);
+      vertex_and_segment<true>(M, S, zoff, Pp, Pc, Pn, i, n, vt, gt, seg, tb, len);
       w.set_vt(i, vt);
       w.set_gt(i, gt);
       finite = finite && isfinite(vt);
@@ -389,8 +381,8 @@ __global__ void __launch_bounds__(128, 4) group_chain_kernel(const ChainParams P
     if (!own) n = 2;
     float L = 0.f, G = 0.f;
     auto refresh_sums = [&]() {
-      L = group_sum_of<kG>(n - 1, gl, [&](int i) { return w.len(i); });
-      if constexpr (kGrad) G = group_sum_of<kG>(n, gl, [&](int i) { return w.gt(i); });
+      L = group_sum_of(n - 1, gl, [&](int i) { return w.len(i); });
+      if constexpr (kGrad) G = group_sum_of(n, gl, [&](int i) { return w.gt(i); });
     };
     refresh_sums();
 
@@ -443,7 +435,7 @@ __global__ void __launch_bounds__(128, 4) group_chain_kernel(const ChainParams P
         float total = 1.f;
         if (some(born)) {
           const float ui = __fadd_rn(__uint_as_float(v23 + 0x3f800000u), -0.999999940395355224609375f);
-          k = group_select<kG>(w, born ? n - 1 : 1, ui, total, gl);
+          k = group_select(w, born ? n - 1 : 1, ui, total, gl);
         }
         // the moved vertex (within), the segment's ends (birth), the removed
         // vertex between its neighbours (death)
@@ -480,9 +472,9 @@ __global__ void __launch_bounds__(128, 4) group_chain_kernel(const ChainParams P
           cs = fminf(fmaxf(cs, -1.0f), 1.0f);
           const float sn = m_sqrt<true>(fmaxf(0.f, (1.0f - cs) * (1.0f + cs)));
           const float sc = __fdividef(gamma, __uint_as_float(hi.x) - cs);
-          const float3 at = birth_point<kGen>(
+          const float3 at = birth_point<true>(
               Af, Bf, sc, __uint_as_float(lo.w) * rh + sn * (__uint_as_float(hi.y) * xi + __uint_as_float(hi.z) * ze),
-              P.birth_fuse_z);
+              false);
           const float tbk = w.tb(k);
           const float ex = R.log_pd - __logf(static_cast<float>(n - 1)) - R.log_pb - __logf(__fdividef(tbk, total));
           if (born) {
@@ -516,7 +508,7 @@ __global__ void __launch_bounds__(128, 4) group_chain_kernel(const ChainParams P
           const float3 Pp = newpos(v - 1);
           const float3 Pn = newpos(v + 1);
           float seg_, tb_, len_;
-          vertex_and_segment<kGen>(M, S, zoff, Pp, Pc, Pn, v, n_new, nvt, ngt, seg_, tb_, len_);
+          vertex_and_segment<true>(M, S, zoff, Pp, Pc, Pn, v, n_new, nvt, ngt, seg_, tb_, len_);
           if (gl < nc - 1) {
             nseg = seg_;
             ntb = tb_;
@@ -531,22 +523,21 @@ __global__ void __launch_bounds__(128, 4) group_chain_kernel(const ChainParams P
             const float2 sl = w.segment(o);
             oseg = sl.x;
             olen = sl.y;
-            if constexpr (kGen) otb = w.tb(o);
-            else otb = w.b * olen;
+            otb = w.tb(o);
           }
         }
         __syncwarp();
         float dlp = (nvt + nseg) - (ovt + oseg);
         dlp += __shfl_xor_sync(kFull, dlp, 1);
         dlp += __shfl_xor_sync(kFull, dlp, 2);
-        dlp = group_get<kG>(dlp, 0);
+        dlp = group_get(dlp, 0);
         if (some(dead)) {
           float dtb = ntb - otb;
           dtb += __shfl_xor_sync(kFull, dtb, 1);
           dtb += __shfl_xor_sync(kFull, dtb, 2);
-          dtb = group_get<kG>(dtb, 0);
-          const float tb_new = group_get<kG>(ntb, 0);
-          const float Tb = group_sum_of<kG>(dead ? n - 1 : 0, gl, [&](int i) { return w.tb(i); });
+          dtb = group_get(dtb, 0);
+          const float tb_new = group_get(ntb, 0);
+          const float Tb = group_sum_of(dead ? n - 1 : 0, gl, [&](int i) { return w.tb(i); });
           const float Tb_red = Tb + dtb;
           if (dead)
             extra = -R.log_pd + __logf(static_cast<float>(n - 2)) + R.log_pb + __logf(__fdividef(tb_new, Tb_red)) + lid;
@@ -590,8 +581,8 @@ __global__ void __launch_bounds__(128, 4) group_chain_kernel(const ChainParams P
             }
           }
           if (accept && gl == 0 && !death) w.set_pos(inew, fnew);
-          dlen = group_get<kG>(dlen, 0);
-          if constexpr (kGrad) dg = group_get<kG>(dg, 0);
+          dlen = group_get(dlen, 0);
+          if constexpr (kGrad) dg = group_get(dg, 0);
           __syncwarp();
           if (accept) {
             A.acc_i += within && !end;
@@ -659,7 +650,7 @@ __global__ void __launch_bounds__(128, 4) group_chain_kernel(const ChainParams P
 }
 
 // The dynamic shared-memory limit and carve-out of a kernel, once per device.
-template <bool kGen, bool kGrad, bool kSpill, int kG>
+template <bool kGrad, bool kSpill>
 cudaError_t group_attributes() {
   static int done[64] = {};
   int dev = 0;
@@ -669,7 +660,7 @@ cudaError_t group_attributes() {
   int optin = 0;
   e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
-  const auto kernel = group_chain_kernel<kGen, kGrad, kSpill, kG>;
+  const auto kernel = group_chain_kernel<kGrad, kSpill>;
   e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
@@ -678,12 +669,12 @@ cudaError_t group_attributes() {
 }
 
 // Launch (blocks_per_sm == nullptr) or occupancy query of one instance.
-template <bool kGen, bool kGrad, bool kSpill, int kG>
+template <bool kGrad, bool kSpill>
 cudaError_t group_call(const ChainParams* p, int grid, int warps_per_block, size_t smem, int* blocks_per_sm,
                        cudaStream_t s) {
-  cudaError_t e = group_attributes<kGen, kGrad, kSpill, kG>();
+  cudaError_t e = group_attributes<kGrad, kSpill>();
   if (e != cudaSuccess) return e;
-  const auto kernel = group_chain_kernel<kGen, kGrad, kSpill, kG>;
+  const auto kernel = group_chain_kernel<kGrad, kSpill>;
   if (blocks_per_sm != nullptr)
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kernel, warps_per_block * 32, smem);
   kernel<<<grid, warps_per_block * 32, smem, s>>>(*p);

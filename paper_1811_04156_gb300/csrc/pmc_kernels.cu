@@ -540,7 +540,7 @@ __global__ void __launch_bounds__(256)
                   const unsigned int slot = atomicAdd(count, 1u);
                   if (slot >= static_cast<unsigned int>(max_paths)) return;
                   float* ox = out_xyz + static_cast<size_t>(slot) * stride;
-                  record_photon<false>(M, S, k0, k1, ph, r_reject, max_scatter, ox, ox + plane, ox + 2 * plane);
+                  record_photon(M, S, k0, k1, ph, r_reject, max_scatter, ox, ox + plane, ox + 2 * plane);
                   out_n[slot] = pr.nsc + 2;
                 });
 }
@@ -757,7 +757,7 @@ __global__ void __launch_bounds__(128) seed_record_kernel(const DMedium M, DPair
   S.org[0] = S.org[1] = S.org[2] = 0.f;  // record frame coordinates
   const uint32_t k0 = static_cast<uint32_t>(seed), k1 = static_cast<uint32_t>(seed >> 32);
   float* gx = xyz + chain_base[c];
-  const PhotonResult pr = record_photon<false>(M, S, k0, k1, sel[i], r_reject, S.cap - 2, gx, gx + S.cap, gx + 2 * S.cap);
+  const PhotonResult pr = record_photon(M, S, k0, k1, sel[i], r_reject, S.cap - 2, gx, gx + S.cap, gx + 2 * S.cap);
   nv[c] = pr.hit ? pr.nsc + 2 : 2;
   status[c] = pr.hit ? 0 : ST_BAD_N;
 }

@@ -213,12 +213,11 @@ __device__ __forceinline__ bool fly_photon(const DMedium& M, const DPair& S, con
 // One photon (index ph) with its vertices (source, scattering points, sensor
 // crossing) recorded to (ox, oy, oz) in absolute coordinates (frame
 // coordinates + S.org).
-template <bool kLean>
 __device__ inline PhotonResult record_photon(const DMedium& M, const DPair& S, uint32_t k0, uint32_t k1,
                                              unsigned long long ph, float r_reject, int max_scatter, float* ox,
                                              float* oy, float* oz) {
   const FlightConsts C(M);
-  Photon p = emit_photon<kLean>(S, k0, k1, ph);
+  Photon p = emit_photon<false>(S, k0, k1, ph);
   PhotonResult res;
   float3 at = p.x;
   for (;;) {
@@ -228,7 +227,7 @@ __device__ inline PhotonResult record_photon(const DMedium& M, const DPair& S, u
       oy[0] = at.y + S.org[1];
       oz[0] = at.z + S.org[2];
     }
-    const bool done = fly_photon<kLean>(M, S, C, k0, k1, ph, r_reject, max_scatter, p, res, at);
+    const bool done = fly_photon<false>(M, S, C, k0, k1, ph, r_reject, max_scatter, p, res, at);
     ox[i + 1] = at.x + S.org[0];
     oy[i + 1] = at.y + S.org[1];
     oz[i + 1] = at.z + S.org[2];

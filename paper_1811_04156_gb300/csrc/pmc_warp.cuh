@@ -1,7 +1,7 @@
 // Pieces shared by the chain kernels that keep a path in a warp's shared memory
-// (pmc_chain.cu: one warp per chain; pmc_group.cu: several chains per warp, or
-// several steps of one chain): the path's arrays, the staged random numbers of
-// a step, and the lane-parallel gradient of a vertex.
+// (pmc_chain.cu: one warp per chain, or a team of warps; pmc_group.cuh: several chains
+// per warp): the path's arrays, the staged random numbers of a step, and the
+// lane-parallel gradient of a vertex.
 #pragma once
 
 #include "pmc_internal.h"
@@ -77,7 +77,7 @@ struct WarpPath {
 // factors that end / start at v, lanes 2-4 the scattering angles at v-1, v,
 // v+1, lane 5 the emission and detection factors; a shuffle tree sums them
 // and every lane returns the total.  Same formulas as grad_vertex.
-template <int kWidth, class PosF>
+template <class PosF>
 __device__ float3 grad_vertex_warp(const DMedium& M, const DPair& S, float zoff, PosF pos, int n, int v, int lane) {
   float3 pv[5];
 #pragma unroll
@@ -157,7 +157,7 @@ __device__ float3 grad_vertex_warp(const DMedium& M, const DPair& S, float zoff,
     g.y += __shfl_xor_sync(kFull, g.y, o);
     g.z += __shfl_xor_sync(kFull, g.z, o);
   }
-  return f3(__shfl_sync(kFull, g.x, 0, kWidth), __shfl_sync(kFull, g.y, 0, kWidth), __shfl_sync(kFull, g.z, 0, kWidth));
+  return f3(__shfl_sync(kFull, g.x, 0), __shfl_sync(kFull, g.y, 0), __shfl_sync(kFull, g.z, 0));
 }
 
 // Point of a birth: mid-point of the foci + sc * t.  In a homogeneous medium the
