@@ -63,9 +63,9 @@ WORKLOAD_TEXT = {
 # csrc/pmc_internal.h, in that order): warp instructions per proposal and DRAM
 # bytes (read + write) of one 65,536-chain x 100,000-step launch (window 20).
 # With another source the bench reports them as null.
-LANE_CAPTURE = {"source_sha256": "13fa0e6016f665450832f73172f44e00669b2c05cc053d9a3582fdd3a355187a",
-                "inst_per_proposal": 37.86, "dram_bytes_per_launch": 83732224.0,
-                "capture": "ncu dram__bytes_read.sum + dram__bytes_write.sum (60.0 MB + 23.7 MB) of one "
+LANE_CAPTURE = {"source_sha256": "fe79a1673cdc3e494086fa3b49abed02463ba12e4eac0ed8c789e7c7ab743605",
+                "inst_per_proposal": 37.86, "dram_bytes_per_launch": 83563264.0,
+                "capture": "ncu dram__bytes_read.sum + dram__bytes_write.sum (60.0 MB + 23.6 MB) of one "
                            "65,536-chain x 100,000-step launch, window 20, 2 warps per CTA"}
 
 

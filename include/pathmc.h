@@ -402,8 +402,9 @@ PMC_API int pmc_total_chains(pmc_chains_t chains);
  * one-past-last position in the processing order, warps per block,
  * persistent grid size, and the kernel: 0 the lean and 1 the general kernel
  * with one warp per chain (or what the autotuner took in its place: 8 lanes of
- * a warp per chain, or the four warps of a block per chain), 2 the general kernel with tree moves, 3 with HMC
- * moves, 4 the lean kernel with one chain per lane (32 chains per warp), 5
+ * a warp per chain, or the four warps of a block per chain; where the paths of
+ * the moment are too long for it, a run takes another of these, with the same
+ * chains), 2 the general kernel with tree moves, 3 with HMC moves, 4 the lean kernel with one chain per lane (32 chains per warp), 5
  * the same with MALA moves, 6 the general kernel sampling the wavelength, 7
  * the lean kernel with tree moves, 8 the lean kernel with one chain per lane
  * and tree moves (each warp's tree moves pooled over its 32 lanes).

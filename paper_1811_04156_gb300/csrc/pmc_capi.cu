@@ -766,7 +766,8 @@ static bool fused_births(pmc_chains_t ch, const ChainClass& cl) {
 // 10.3 ms with one warp per chain (window 256), 6.9 ms in groups (window 128;
 // 8.4 with 96, 9.3 with 192; 6.2 flushing subnormals).  Paths grow longer than the
 // straight line's, so each launch may take a warp per chain instead (set_choices).
-// The lean kernel's longer paths spill there (40 against 30 ms).  Teams: offered to the autotuner up to four chains per SM
+// The lean kernel's longer paths spill there (40 against 30 ms).
+// Teams: offered to the autotuner up to four chains per SM
 // (one warp per scheduler); 1,000 plain steps of 64 chains 0.94 ms with one warp
 // per chain, 0.75 with teams, of 608 chains 0.96 and 0.93, of 912 1.01 and 1.57
 // (100 layers: 1.39 and 1.16, 1.41 and 1.45, 1.49 and 2.55).
@@ -991,10 +992,11 @@ static int set_choices(pmc_chains_t ch) {
     auto add = [&](int share, bool spill, int window, int wpb) -> cudaError_t {
       int bps = 0;
       const cudaError_t e = ch->kernels->occupancy(cl.kind, share, ch->grad, spill, wpb, window, &bps);
-      if (e == cudaSuccess && bps >= 1)
-        cl.others.push_back({share, spill, window, wpb,
-                             std::max(1, std::min((work_items(cl.kind, share, chains) + wpb - 1) / wpb, bps * ch->ctx->n_sm))});
-      return e;
+      if (e != cudaSuccess) return e;
+      if (bps < 1) return cudaErrorInvalidConfiguration;  // (an option without a kernel would step no chain)
+      cl.others.push_back({share, spill, window, wpb,
+                           std::max(1, std::min((work_items(cl.kind, share, chains) + wpb - 1) / wpb, bps * ch->ctx->n_sm))});
+      return cudaSuccess;
     };
     if (cl.kind < 2 && cl.share == 0 && cl.spill) {
       cl.rule = {{cl.smem_cap - 1, cl.smem_cap - 1}, {chains / kBeyondShare, INT_MAX}};

@@ -34,9 +34,9 @@ struct BatchPos {
 // because its path is shorter than a warp; a path's terms meet again in
 // shared memory.
 //
-// Bound by instruction issue (340 warp instructions per 32 vertices, 77 % issue,
+// Bound by instruction issue (304 warp instructions per 32 vertices, 78 % issue,
 // against 12 bytes per vertex).  One warp per path ran at 16.6 active lanes on
-// paths of 21 vertices: 131,072 paths (cap 64) took 60 us, in tiles 33 us.
+// paths of 21 vertices: 131,072 paths (cap 64) took 60 us, in tiles 31 us.
 // ---------------------------------------------------------------------------
 constexpr int kTile = 128;          // threads of a block
 constexpr int kTileItems = 1024;    // vertices whose terms a block holds at once
